@@ -53,6 +53,18 @@ struct FftGroup {
 };
 #define TL_MAX_FFT_GROUPS 24
 
+// Ring groups of the single-precision synthesis kernels (ringsynth.cu): mode and log2 of
+// the transform length, rings sy_rings[first .. first + count), largest band of them.
+struct SyGroup {
+  int mode, lg, first, count, band;
+};
+#define TL_MAX_SY_GROUPS 16
+constexpr int kSyCorr = 5120;  // entries of each window's correction table
+// interpolation window: per tap of the first half, the polynomial's coefficients in s
+struct SyWindow {
+  float c10[5][9], c8[4][9];
+};
+
 }  // namespace tl
 
 struct tl_plan {
@@ -73,10 +85,18 @@ struct tl_plan {
   int blue_reg_lg;      // Bluestein lengths M >= 2^blue_reg_lg (up to 2^12) run the register passes and keep
                         // their spectra in natural order (0: none; bit-reversed order for the others)
   int fft_batch;        // Bluestein sub-transforms run together in the ring FFT (1 or 4; 0 = choose)
-  int ring_reg;         // single precision: register-pass ring FFT where a group allows it (1, default) or not (0)
+  int ring_reg;         // single precision: the synthesis kernels of ringsynth.cu (1, default) or the general one (0)
   int *fft_rings;       // ring indices grouped by FFT launch (device)
   int fft_ngroups;
   tl::FftGroup fft_groups[TL_MAX_FFT_GROUPS];
+  // single-precision ring synthesis: its groups, and those of the rings it does not take
+  int sy_ngroups, rest_ngroups;
+  tl::SyGroup sy_groups[TL_MAX_SY_GROUPS];
+  int4 *sy_rings;       // {ring, band, fold, 0} by group (device)
+  float *sy_corr;       // [2][kSyCorr] corrections of the two windows (device)
+  tl::SyWindow sy_win;
+  int *rest_rings;      // ring indices of rest_groups (device)
+  tl::FftGroup rest_groups[TL_MAX_FFT_GROUPS];
   // workspace
   void *tab0, *tab2;    // plan-time step tables {k_l, A_{l+1}} for spin 0 and spin 2
   void *rec_T, *rec_P, *rec_QU; // coefficient records
@@ -237,7 +257,17 @@ void host_twiddles(int TW, double *tw);
 size_t ringfft_smem_bytes(const tl_plan *p);
 // ring-FFT launch groups (no allocation): fills groups[] and order[nrings]; returns
 // the number of groups, or -1 if there are more than TL_MAX_FFT_GROUPS
-int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGroup *groups, int *order);
+// (of the rings with use[r] != 0 only, when use is given)
+int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGroup *groups, int *order,
+                    const unsigned char *use = nullptr);
+// mcut[r]: the largest m whose coefficients can be non-zero on ring r at band limit lmax
+void host_ring_bands(int nside, int lmax, const double *sint, const double *z, int *mcut);
+struct JobList;
+void host_synth_window(SyWindow *w, float *corr10, float *corr8);
+int host_synth_groups(int nside, int nrings, const int *nphi, const int *mcut, SyGroup *groups, int4 *rings, int *rest,
+                      int *nrest);
+cudaError_t launch_ring_synth(const tl_plan *p, const JobList &jl, cudaStream_t s);
+cudaError_t raise_smem(const void *fn, size_t bytes);
 cudaError_t launch_bluestein_setup_impl(tl_plan *p, const double2 *tw64, cudaStream_t s);
 
 // normalisation of theta derivatives inside the Legendre stage: lambda^(j) / L^j

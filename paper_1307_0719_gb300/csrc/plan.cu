@@ -101,7 +101,7 @@ static void free_plan(tl_plan *p) {
                   p->tc_blk0, p->tc_blk2, p->tc_bm0, p->tc_bm2, p->tc_step0, p->tc_step2, p->tc_b0, p->tc_bp, p->tc_b2, p->dev_err,
                   p->tc_bs0, p->tc_bsp, p->tc_bs2, p->tc_st0, p->tc_stp, p->tc_st2, p->tc_sm0, p->tc_smp,
                   p->tc_sm2,
-                  p->fft_rings};
+                  p->fft_rings, p->sy_rings, p->sy_corr, p->rest_rings};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   if (p->timing)
@@ -159,8 +159,35 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
     TRY_CUDA(upload(&p->fft_rings, order, B));
   }
 
+  // the single-precision ring synthesis: the ring groups of its grids
+  const char *rr = getenv("TAYLENS_RING_FFT");  // "shared": the general kernel for every ring
+  p->ring_reg = (rr && strcmp(rr, "shared") == 0) ? 0 : 1;
+  int sy_tw = 0;
+  if (precision != TL_FP64 && p->ring_reg) {
+    std::vector<int> mcut(p->nrings), rest(p->nrings), order(p->nrings);
+    std::vector<int4> rings(p->nrings);
+    host_ring_bands(nside, lmax, h.sint.data(), h.z.data(), mcut.data());
+    int nrest = 0;
+    p->sy_ngroups = host_synth_groups(nside, p->nrings, h.nphi.data(), mcut.data(), p->sy_groups, rings.data(),
+                                      rest.data(), &nrest);
+    if (nrest > 0) {
+      std::vector<unsigned char> use(p->nrings, 0);
+      for (int i = 0; i < nrest; ++i) use[rest[i]] = 1;
+      p->rest_ngroups = host_fft_groups(nside, p->nrings, h.nphi.data(), ml.data(), p->rest_groups, order.data(),
+                                        use.data());
+      if (p->rest_ngroups < 0) return TL_ERR_UNSUPPORTED;
+      TRY_CUDA(upload(&p->rest_rings, order, B));
+    }
+    std::vector<float> corr(2 * (size_t)kSyCorr);
+    host_synth_window(&p->sy_win, corr.data(), corr.data() + kSyCorr);
+    TRY_CUDA(upload(&p->sy_rings, rings, B));
+    TRY_CUDA(upload(&p->sy_corr, corr, B));
+    for (int i = 0; i < p->sy_ngroups; ++i) sy_tw = sy_tw > (4 << p->sy_groups[i].lg) ? sy_tw : (4 << p->sy_groups[i].lg);
+  }
+
   // twiddles e^{-2 pi i k / TW}, k < TW/2, for every power-of-two length used
-  const int TW = host_twiddle_len(nside, maxm);
+  int TW = host_twiddle_len(nside, maxm);
+  while (TW < sy_tw) TW <<= 1;
   p->tw_len = TW;
   std::vector<double> tw64(TW);  // interleaved (re, im)
   host_twiddles(TW, tw64.data());
@@ -179,8 +206,6 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
   }
   TRY_CUDA(dalloc(&p->phase, e2 * phase_table_entries(nside), B));
   TRY_CUDA(launch_phase_table(p, p->phase, 0));
-  const char *rr = getenv("TAYLENS_RING_FFT");  // "shared": the shared-memory kernel for every group
-  p->ring_reg = (rr && strcmp(rr, "shared") == 0) ? 0 : 1;
   p->blue_reg_lg = (precision != TL_FP64 && p->ring_reg) ? 11 : 0;
   cudaError_t e = launch_bluestein_setup_impl(p, (const double2 *)dtw64, 0);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -354,12 +379,17 @@ extern "C" tl_status tl_plan_set_wait_limit(tl_plan *p, int polls, int stall) {
 extern "C" int tl_plan_maps_per_field(const tl_plan *p) { return p ? p->nmaps : 0; }
 extern "C" int tl_plan_batch(const tl_plan *p) { return p ? p->batch : 0; }
 
+// launches of one launch_ringfft call: one per ring group
+static long long ring_launches(const tl_plan *p) {
+  return p->sy_ngroups > 0 ? p->sy_ngroups + p->rest_ngroups : p->fft_ngroups;
+}
+
 extern "C" long long tl_plan_batch_launches(const tl_plan *p, int nreal, int with_phi) {
   if (!p || nreal < 0) return -1;
   const bool pol = (p->spins & TL_SPIN_QU) != 0;
-  const long long G = p->fft_ngroups;  // one ring-FFT launch per ring group
+  const long long G = ring_launches(p);  // ring-FFT launches of one realisation's maps
   // a potential with its own band limit: prep, Legendre and FFT on its plan per realisation
-  const long long sub = (with_phi && p->phi_plan) ? 2 + p->phi_plan->fft_ngroups : 0;
+  const long long sub = (with_phi && p->phi_plan) ? 2 + ring_launches(p->phi_plan) : 0;
   const bool phi = with_phi != 0 && !p->phi_plan;
   if (p->batch > 1) {
     // per batch: coefficient tiles and Legendre launch of T, the potential and Q/U

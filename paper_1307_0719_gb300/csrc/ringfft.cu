@@ -13,36 +13,15 @@
 // memory; the chirp spectra of Bluestein are tabulated per length at plan time.
 #include <math.h>
 
+#include <algorithm>
+#include <mutex>
+
 #include "fft.cuh"
 #include "regfft.cuh"
+#include "ringjobs.cuh"
 
 namespace tl {
 
-// One output map: its coefficient plane's first ring (T2 [ring][m], chosen on the
-// host, so that the kernel indexes no parameter array at run time), phi-derivative
-// order k, 1/sin(theta) weight and output scale (double, and rounded to float).
-struct JobDev {
-  const void *in;
-  void *out;
-  double scale;
-  float scalef;
-  int k, div_sint;
-  long long tile;  // output layout: 0 plain, else the tile stride (see d3_pix)
-  int il;          // input rows four-ring interleaved (element m at row[4 m])
-};
-
-// The ring's coefficient row in a plane and the element stride along m
-template <typename T2>
-__device__ __forceinline__ const T2 *job_row(const JobDev &J, int r, int mmax, int &fs) {
-  fs = J.il ? 4 : 1;
-  return J.il ? (const T2 *)J.in + (size_t)(r >> 2) * (size_t)(mmax + 1) * 4 + (r & 3)
-              : (const T2 *)J.in + (size_t)r * (mmax + 1);
-}
-#define TL_MAX_JOBS 96
-struct JobList {
-  int n;
-  JobDev job[TL_MAX_JOBS];
-};
 // adjoint: one output plane (plane 0..2 = T, Q, U with inputs d_theta^j d_phi^k,
 // k < nk, at base + map_index(j, k) npix; plane 3 = phi with one input map at base),
 // written at fout (T2 [ring][m], its first ring)
@@ -80,19 +59,6 @@ static int ring_sub_stride_max(const FftGroup &g) {
 template <typename T> __device__ __forceinline__ T scale2(T x, int n);
 template <> __device__ __forceinline__ float scale2<float>(float x, int n) { return scalbnf(x, n); }
 template <> __device__ __forceinline__ double scale2<double>(double x, int n) { return scalbn(x, n); }
-
-// (i)^k g
-template <typename T2>
-__device__ __forceinline__ T2 rot_ik(T2 a, int k) {
-  T2 g;
-  switch (k & 3) {
-    case 0: g = a; break;
-    case 1: g.x = -a.y; g.y = a.x; break;
-    case 2: g.x = -a.x; g.y = -a.y; break;
-    default: g.x = a.y; g.y = -a.x; break;
-  }
-  return g;
-}
 
 // The class sum for the two jobs of a transform in one pass over the class's m: the
 // weight, the sign and the power (m/L)^k (built once up to the larger k) are
@@ -193,25 +159,11 @@ __device__ __forceinline__ void reg_bluestein(float2 *Y, int SY, int ni, float2 
 }
 
 // BLUE: the launch's rings have non-power-of-two sub-transforms (Bluestein); else
-// power-of-two ones. REG: Bluestein by register passes (reg_bluestein; see ring_threads). A launch covers one ring group, so each instance carries one
-// sub-transform path (and its own register allocation). LG > 0: the group's
-// transform length is known at compile time, 2^LG (power-of-two rings: the
-// sub-transform length ni; Bluestein: the convolution length M), so the FFT's index
-// and address arithmetic folds into constants; LG = 0 takes it from the ring.
-// threads of a ring-FFT CTA: 256 for the register Bluestein (M = 2^12: one
-// sub-transform at a time, 100 KB of shared memory, two CTAs per SM at 128 registers;
-// M = 2^11: two at a time, 68 KB, three CTAs per SM), so that the CTAs' phases
-// (fold from HBM, transforms, output pass) interleave; else 512
-template <bool REG, int LG> constexpr int ring_threads() { return (REG && LG >= 11) ? 256 : 512; }
-// CTAs per SM the register allocation is held to: M = 2^11 fits three (68 KB of shared
-// memory each), M = 2^12 two
-template <typename T, bool REG, int LG> constexpr int ring_min_ctas() {
-  return sizeof(T) != 4 ? 1 : (REG && LG == 11) ? 3 : 2;
-}
-
-template <typename T, bool BLUE, int LG = 0, bool REG = false>
-__global__ void __launch_bounds__(ring_threads<REG, LG>(), ring_min_ctas<T, REG, LG>()) ringfft_kernel(RingTable rt, int nside, int mmax, JobList jobs,
-                                                      BluesteinTable bt,
+// power-of-two ones. A launch covers one ring group, so each instance carries one
+// sub-transform path (and its own register allocation).
+template <typename T, bool BLUE>
+__global__ void __launch_bounds__(512, (sizeof(T) == 4 ? 2 : 1)) ringfft_kernel(RingTable rt, int nside, int mmax,
+                                                      JobList jobs, BluesteinTable bt,
                                                       const typename RealTraits<T>::T2 *__restrict__ tw, int TW,
                                                       int bbatch, T invL, const int *__restrict__ rings,
                                                       const typename RealTraits<T>::T2 *__restrict__ phase) {
@@ -221,8 +173,7 @@ __global__ void __launch_bounds__(ring_threads<REG, LG>(), ring_min_ctas<T, REG,
   const int pair = blockIdx.y;
   const int ja = 2 * pair, jb = 2 * pair + 1;
   const bool hasb = jb < jobs.n;
-  constexpr bool LGP = LG > 0 && !BLUE;  // power-of-two rings of one known length
-  const int N = LGP ? (4 << LG) : rt.nphi[r];
+  const int N = rt.nphi[r];
   const int ni = N >> 2;
   const int half = N >> 1;
   const long long first = rt.first[r];
@@ -232,8 +183,8 @@ __global__ void __launch_bounds__(ring_threads<REG, LG>(), ring_min_ctas<T, REG,
   // FFT); other ni: plain, with SY = 4 mod 16 so that the four arrays fall on
   // different banks.
   const bool pw2 = !BLUE;  // the group is of one kind: (ni & (ni - 1)) == 0 iff !BLUE
-  const int lgni = LGP ? LG : 31 - __clz(ni);
-  const int SY = LGP ? (1 << LG) : ring_sub_stride(ni);
+  const int lgni = 31 - __clz(ni);
+  const int SY = ring_sub_stride(ni);
   T2 *Y = (T2 *)smem_raw;
   T2 *W = Y + 4 * SY;  // work area
   const bool yswz = pw2 && ni >= 16;  // the XOR layout needs whole 16-element blocks
@@ -407,24 +358,20 @@ __global__ void __launch_bounds__(ring_threads<REG, LG>(), ring_min_ctas<T, REG,
   // ---- four length-ni inverse DFTs
   if (!BLUE) {
     if (yswz)
-      fft_core<true, T, T2, LGP ? LG : 0>(Y, ni, 4, SY, +1, tw, TW);
+      fft_core<true, T, T2>(Y, ni, 4, SY, +1, tw, TW);
     else
-      fft_core<false, T, T2, LGP ? LG : 0>(Y, ni, 4, SY, +1, tw, TW);
-  } else if constexpr (REG) {
-    reg_bluestein<LG, ring_threads<REG, LG>()>((float2 *)Y, SY, ni, (float2 *)W,
-                                               (const float2 *)bt.spec + bt.offset[ni], (const float2 *)tw,
-                                               31 - __clz(TW));
+      fft_core<false, T, T2>(Y, ni, 4, SY, +1, tw, TW);
   } else {
     const long long off = bt.offset[ni];
-    const int M = LG ? (1 << LG) : bt.mlen[ni];
+    const int M = bt.mlen[ni];
     const T2 *bh = (const T2 *)bt.spec + off;
     const T2 *ch = bh + M;  // the length's chirp follows its spectrum
     const int SW = M;
     if (bbatch >= 4) {
-      bluestein_batch<T, T2, LG>(Y, ni, SY, M, 4, W, SW, bh, ch, tw, TW);
+      bluestein_batch<T, T2>(Y, ni, SY, M, 4, W, SW, bh, ch, tw, TW);
     } else {
       for (int t2 = 0; t2 < 4; ++t2)
-        bluestein_batch<T, T2, LG>(Y + t2 * SY, ni, SY, M, 1, W, SW, bh, ch, tw, TW);
+        bluestein_batch<T, T2>(Y + t2 * SY, ni, SY, M, 1, W, SW, bh, ch, tw, TW);
     }
   }
 
@@ -461,202 +408,6 @@ __global__ void __launch_bounds__(ring_threads<REG, LG>(), ring_min_ctas<T, REG,
       outB[oidx(JB.tile, p1 + 2 * ni)] = sb * X2.y;
       outB[oidx(JB.tile, p1 + 3 * ni)] = sb * X3.y;
     }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Rings of N = 2^LG pixels without aliasing (N > mmax), single precision: one CTA of
-// N / 16 threads per (ring, pair of output maps). The fold is formed straight in the
-// registers of the first FFT pass (thread h, slot c: Z_t with t = h + (N/16) c), the
-// register passes of RegFft run the inverse DFT, and each thread stores its sixteen
-// outputs. Per output class t, with class t holding m1 = t and class N - t holding
-// m2 = N - t (m2 = 0 for t = 0), each present when m <= mmax:
-//   Z_t = e_t [ u_a p_a(m1) F^a_m1 + u_b p_b(m1) F^b_m1
-//               + sigma conj(u_a p_a(m2) F^a_m2 - u_b p_b(m2) F^b_m2) ],
-// u_a = w_a i^k_a / 2, u_b = i w_b i^k_b / 2 (w: the job's 1/sin(theta) weight and
-// balance), p(m) = w_m (m / L)^k, e_t = e^{i pi t / N} and sigma = -1 on
-// half-pixel-shifted rings (t > 0), e_t = sigma = 1 otherwise: the class sums and
-// the Hermitian split of the shared-memory kernel above, written per class.
-template <int LG>
-__global__ void __launch_bounds__(1 << (LG - 4), 1024 >> (LG - 4))
-    ringfft_reg_kernel(RingTable rt, int mmax, JobList jobs, const float2 *__restrict__ tw, int lgtw, float invL,
-                       const int *__restrict__ rings, const float2 *__restrict__ phase) {
-  typedef RegFft<LG, +1> F;
-  constexpr int N = F::N, TG = F::TG, HALF = N / 2;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2 *sm = (float2 *)smem_raw;
-  const int r = rings[blockIdx.x];
-  const int pair = blockIdx.y, ja = 2 * pair, jb = 2 * pair + 1;
-  const bool hasb = jb < jobs.n;
-  const int h = threadIdx.x;
-  const long long first = rt.first[r];
-  const bool shifted = __double_as_longlong(rt.phi0[r]) != 0;
-  const JobDev JA = jobs.job[ja];
-  const JobDev JB = hasb ? jobs.job[jb] : jobs.job[ja];
-  int fs;
-  const float2 *FA = job_row<float2>(JA, r, mmax, fs);
-  const float2 *FB = job_row<float2>(JB, r, mmax, fs);
-  const bool same = JA.in == JB.in;
-  const float inv_s = rt.rsinf[r];
-  float wa = JA.div_sint ? inv_s : 1.0f;
-  float wb = hasb ? (JB.div_sint ? inv_s : 1.0f) : 0.0f;
-  float sa = JA.scalef, sb = JB.scalef;
-  {  // magnitude balance of the packed maps, as in ringfft_kernel
-    const float Lf = 1.0f / invL, sf = rt.ringf[8 * (size_t)r + 1];
-    const int e = max(0, __float2int_rn(log2f(Lf / (1.0f + Lf * sf))));
-    const int ea = e * max(0, JA.k - JA.div_sint), eb = e * max(0, JB.k - JB.div_sint);
-    wa = scalbnf(wa, ea);
-    wb = scalbnf(wb, eb);
-    sa = scalbnf(sa, -ea);
-    sb = scalbnf(sb, -eb);
-  }
-  const int kA = JA.k, kB = hasb ? JB.k : 0;
-  const int klo = min(kA, kB), khi = max(kA, kB);
-  const float2 ua = rot_ik(f2(0.5f * wa, 0.0f), kA);
-  const float2 ub = rot_ik(f2(0.5f * wb, 0.0f), kB + 1);
-  const float2 *__restrict__ eph = phase + ((size_t)(N / 4) * (N / 4) - 1);  // e^{i pi t / N}, t <= N/2
-
-  // w_m (m / L)^k for the two jobs: binary powers (k <= 7), no loops
-  auto powers = [&](int m, float &pa, float &pb) {
-    const float m1 = (float)m * invL, m2 = m1 * m1, m4 = m2 * m2;
-    const float w = (m > 0) ? 2.0f : 1.0f;
-    pa = w;
-    pb = w;
-    if (kA & 1) pa *= m1;
-    if (kA & 2) pa *= m2;
-    if (kA & 4) pa *= m4;
-    if (kB & 1) pb *= m1;
-    if (kB & 2) pb *= m2;
-    if (kB & 4) pb *= m4;
-  };
-  // u_a p_a(m) F^a_m + s u_b p_b(m) F^b_m (s = +1: the class's own term; -1 inside
-  // the conjugate of the partner class's term)
-  auto comb = [&](int m, float2 fa, float2 fb, float s) -> float2 {
-    float pa, pb;
-    powers(m, pa, pb);
-    const float2 ta = cmul(ua, f2(pa * fa.x, pa * fa.y));
-    const float2 tb = cmul(ub, f2(pb * fb.x, pb * fb.y));
-    return f2(fmaf(s, tb.x, ta.x), fmaf(s, tb.y, ta.y));
-  };
-  const float sg = shifted ? -1.0f : 1.0f;  // sigma of the classes t > 0
-  const float2 zero = f2(0.0f, 0.0f);
-  float2 x[16];
-  if (mmax <= HALF && same) {
-    // Slot c < 8 (t < N/2) holds class t's own term only, slot c >= 8 (t >= N/2) the
-    // conjugate of class N - t's only: one coefficient per slot (both maps read one
-    // plane), all sixteen loads in flight before the arithmetic, which then runs in
-    // place. Classes 0 and N/2 get their other term below.
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int t = h + TG * c;
-      const int m = c < 8 ? t : N - t;
-      x[c] = m <= mmax ? __ldg(FA + (size_t)m * fs) : zero;
-    }
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int t = h + TG * c;
-      if (c < 8) {
-        x[c] = comb(t, x[c], x[c], 1.0f);
-      } else {
-        const float2 d = comb(N - t, x[c], x[c], -1.0f);
-        x[c] = f2(sg * d.x, -sg * d.y);
-      }
-    }
-    if (h == 0) {
-      const float2 f0 = __ldg(FA);
-      const float2 d0 = comb(0, f0, f0, -1.0f);
-      x[0] = f2(x[0].x + d0.x, x[0].y - d0.y);
-      if (HALF <= mmax) {
-        const float2 fa = __ldg(FA + (size_t)HALF * fs);
-        x[8] = cadd(x[8], comb(HALF, fa, fa, 1.0f));
-      }
-    }
-  } else if (mmax <= HALF) {
-    // as above with two coefficient rows: two batches of eight slots
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      float2 va[8], vb[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int t = h + TG * (8 * half + u);
-        const int m = half ? N - t : t;
-        const bool ok = m <= mmax;
-        va[u] = ok ? __ldg(FA + (size_t)m * fs) : zero;
-        vb[u] = (ok && !same) ? __ldg(FB + (size_t)m * fs) : va[u];
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int t = h + TG * (8 * half + u);
-        if (half == 0) {
-          x[u] = comb(t, va[u], vb[u], 1.0f);
-        } else {
-          const float2 d = comb(N - t, va[u], vb[u], -1.0f);
-          x[8 + u] = f2(sg * d.x, -sg * d.y);
-        }
-      }
-    }
-    if (h == 0) {
-      // t = 0: the partner class is class 0 itself (sigma = +1)
-      const float2 d0 = comb(0, __ldg(FA), same ? __ldg(FA) : __ldg(FB), -1.0f);
-      x[0] = f2(x[0].x + d0.x, x[0].y - d0.y);
-      // t = N/2: class N/2's own term m = N/2
-      if (HALF <= mmax) {
-        const float2 fa = __ldg(FA + (size_t)HALF * fs);
-        x[8] = cadd(x[8], comb(HALF, fa, same ? fa : __ldg(FB + (size_t)HALF * fs), 1.0f));
-      }
-    }
-  } else {
-    // band limit above N/2: both terms wherever m <= mmax
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int t = h + TG * c;
-      const int m2 = t ? N - t : 0;
-      float2 z = zero;
-      if (t <= mmax) {
-        const float2 fa = __ldg(FA + (size_t)t * fs);
-        z = comb(t, fa, same ? fa : __ldg(FB + (size_t)t * fs), 1.0f);
-      }
-      if (m2 <= mmax) {
-        const float2 fa = __ldg(FA + (size_t)m2 * fs);
-        const float2 d = comb(m2, fa, same ? fa : __ldg(FB + (size_t)m2 * fs), -1.0f);
-        const float s2 = t ? sg : 1.0f;
-        z.x = fmaf(s2, d.x, z.x);
-        z.y = fmaf(-s2, d.y, z.y);
-      }
-      x[c] = z;
-    }
-  }
-  if (shifted) {
-    // e_t = e^{i pi t / N} = e_h e^{i pi c / 16} (t = h + (N/16) c)
-    // cos, sin of pi c / 16
-    constexpr float kc[16] = {1.00000000000000000000f, 0.98078528040323043058f, 0.92387953251128673848f, 0.83146961230254523567f, 0.70710678118654757274f, 0.55557023301960228867f, 0.38268343236508983729f, 0.19509032201612833135f, 0.00000000000000006123f, -0.19509032201612819257f, -0.38268343236508972627f, -0.55557023301960195560f, -0.70710678118654746172f, -0.83146961230254534669f, -0.92387953251128673848f, -0.98078528040323043058f};
-    constexpr float ks[16] = {0.00000000000000000000f, 0.19509032201612824808f, 0.38268343236508978178f, 0.55557023301960217765f, 0.70710678118654746172f, 0.83146961230254523567f, 0.92387953251128673848f, 0.98078528040323043058f, 1.00000000000000000000f, 0.98078528040323043058f, 0.92387953251128673848f, 0.83146961230254545772f, 0.70710678118654757274f, 0.55557023301960217765f, 0.38268343236508989280f, 0.19509032201612860891f};
-    const float2 eh = __ldg(eph + h);
-#pragma unroll
-    for (int c = 0; c < 16; ++c) x[c] = cmul(x[c], cmul(eh, f2(kc[c], ks[c])));
-  }
-  F::run(x, sm, h, tw, lgtw);
-  float *outA = (float *)JA.out;
-  float *outB = hasb ? (float *)JB.out : nullptr;
-  const long long tile = JA.tile;  // one layout for every job of a launch
-  // The ring starts a tile (the host launches this kernel only for such rings), so
-  // pixel h + TG c sits in tile first / 256 + (h + TG c) / 256 at (h + TG c) mod 256.
-  // For TG >= 256 that is tile (h / 256) + (TG / 256) c at h mod 256; for TG < 256,
-  // h + TG (c mod 256/TG) < 256, so it is tile (TG c) / 256 at h + TG (c mod 256/TG).
-  // Plain maps: first + h + TG c.
-  constexpr int PER = TG >= kD3Tile ? 1 : kD3Tile / TG;
-  const long long base =
-      tile ? ((first >> kD3TileLg) + (TG >= kD3Tile ? (h >> kD3TileLg) : 0)) * tile +
-                 (TG >= kD3Tile ? (h & (kD3Tile - 1)) : h)
-           : first + h;
-  float *oa = outA + base;
-  float *ob = hasb ? outB + base : nullptr;
-#pragma unroll
-  for (int c = 0; c < 16; ++c) {
-    const long long off =
-        tile ? (long long)((TG * c) >> kD3TileLg) * tile + (TG >= kD3Tile ? 0 : TG * (c % PER)) : (long long)TG * c;
-    oa[off] = sa * x[c].x;
-    if (hasb) ob[off] = sb * x[c].y;
   }
 }
 
@@ -959,18 +710,13 @@ static bool group_reg_blue(const tl_plan *p, const FftGroup &g) {
   const int lgM = 31 - __builtin_clz((unsigned)g.M);
   return lgM >= p->blue_reg_lg && lgM <= 12;
 }
-// threads of a group's CTA (ring_threads of its kernel instance)
-static int group_threads(const tl_plan *p, const FftGroup &g) {
-  return (group_reg_blue(p, g) && g.M >= 2048) ? 256 : 512;
-}
-// threads: the CTA size of the kernel that runs the group (group_threads for the
-// forward kernels; 512 for the adjoint), which sets how many register Bluestein
-// sub-transforms run at once, each with its own exchange array
-static size_t group_smem(const tl_plan *p, const FftGroup &g, int batch, int threads) {
+// reg: the kernel runs the group's sub-transforms by register passes (the adjoint, where
+// the plan keeps their spectra in natural order), 512 threads' worth of exchange arrays
+static size_t group_smem(const tl_plan *p, const FftGroup &g, int batch, bool reg) {
   const size_t e2 = (p->precision == TL_FP64) ? 16 : 8;
   const size_t fold = (2 * g.ni_min + 1 < 512) ? 1024 : 0;
-  if (group_reg_blue(p, g)) {  // Y, then one padded exchange array per concurrent sub-transform
-    const size_t k = (size_t)threads / ((size_t)g.M / 16);
+  if (reg && group_reg_blue(p, g)) {  // Y, then one padded exchange array per concurrent sub-transform
+    const size_t k = (size_t)512 / ((size_t)g.M / 16);
     size_t wl = (k < 4 ? k : 4) * ((size_t)g.M + (size_t)g.M / 16);
     if (wl < fold) wl = fold;
     return e2 * ((size_t)4 * ring_sub_stride_max(g) + wl);
@@ -981,9 +727,9 @@ static size_t group_smem(const tl_plan *p, const FftGroup &g, int batch, int thr
 }
 // Four sub-transforms at once when two CTAs still fit on an SM (or when asked to and
 // one fits); one at a time otherwise.
-static int group_batch(const tl_plan *p, const FftGroup &g) {
-  if (g.M == 0 || p->fft_batch == 1 || group_reg_blue(p, g)) return 1;
-  const size_t s4 = group_smem(p, g, 4, 512);
+static int group_batch(const tl_plan *p, const FftGroup &g, bool reg) {
+  if (g.M == 0 || p->fft_batch == 1 || (reg && group_reg_blue(p, g))) return 1;
+  const size_t s4 = group_smem(p, g, 4, reg);
   if (p->fft_batch == 4) return s4 <= 227 * 1024 ? 4 : 1;
   return s4 <= 113 * 1024 ? 4 : 1;
 }
@@ -995,65 +741,16 @@ size_t ringfft_smem_bytes(const tl_plan *p) {
   return e2 * ((size_t)4 * ((size_t)p->nside + 16) + wl);
 }
 
-template <typename K>
-static cudaError_t set_group_smem(const tl_plan *p, K kernel) {
-  size_t mx = 0;
-  for (int i = 0; i < p->fft_ngroups; ++i) {
-    const size_t sm = group_smem(p, p->fft_groups[i], group_batch(p, p->fft_groups[i]), 512);
-    if (sm > mx) mx = sm;
-  }
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
-}
-
-template <typename T>
-using RingKernel = void (*)(RingTable, int, int, JobList, BluesteinTable, const typename RealTraits<T>::T2 *, int,
-                            int, T, const int *, const typename RealTraits<T>::T2 *);
-
-// The kernel instance of a ring group: single precision has compile-time lengths for
-// the belt (sub-transforms of 2^8 .. 2^11, Nside 256 .. 2048) and the larger Bluestein
-// groups (M = 2^9 .. 2^12); every other group, and double precision, the generic one.
-template <typename T>
-static RingKernel<T> pick_ring_kernel(const tl_plan *p, const FftGroup &g) {
-  if constexpr (sizeof(T) == 4) {
-    const int lgM = g.M ? 31 - __builtin_clz((unsigned)g.M) : 0;
-    const int lgn = (g.ni_min == g.ni_max && g.ni_min > 0) ? 31 - __builtin_clz((unsigned)g.ni_min) : 0;
-    if (g.M && group_reg_blue(p, g)) {
-      switch (lgM) {
-        case 11: return ringfft_kernel<T, true, 11, true>;
-        case 12: return ringfft_kernel<T, true, 12, true>;
-        default: break;
-      }
-    }
-    if (g.M) {
-      switch (lgM) {
-        case 9: return ringfft_kernel<T, true, 9>;
-        case 10: return ringfft_kernel<T, true, 10>;
-        case 11: return ringfft_kernel<T, true, 11>;
-        case 12: return ringfft_kernel<T, true, 12>;
-        default: break;
-      }
-    } else if (lgn && (1 << lgn) == g.ni_min) {
-      switch (lgn) {
-        case 8: return ringfft_kernel<T, false, 8>;
-        case 9: return ringfft_kernel<T, false, 9>;
-        case 10: return ringfft_kernel<T, false, 10>;
-        case 11: return ringfft_kernel<T, false, 11>;
-        default: break;
-      }
-    }
-  }
-  return g.M ? ringfft_kernel<T, true, 0> : ringfft_kernel<T, false, 0>;
-}
-
 // Raise a kernel's dynamic shared-memory limit on the current device to what a launch
-// needs, once (kept per kernel and device; host-side, not thread-safe, as the rest
-// of a plan's launches).
-static cudaError_t raise_smem(const void *fn, size_t bytes) {
+// needs, once (kept per kernel and device; plans of several host threads may get here at once).
+cudaError_t raise_smem(const void *fn, size_t bytes) {
   constexpr int kMax = 128;
+  static std::mutex mu;
   static const void *keys[kMax];
   static int devs[kMax];
   static size_t vals[kMax];
   static int nk = 0;
+  std::lock_guard<std::mutex> lock(mu);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -1069,31 +766,6 @@ static cudaError_t raise_smem(const void *fn, size_t bytes) {
   }
   if (i < kMax) vals[i] = bytes;
   return cudaSuccess;
-}
-
-// The register-pass kernel of a ring group, or nullptr: single precision, rings of
-// one power-of-two length N = 4 ni = 2^LG (LG 10 .. 13) without aliasing (N > mmax),
-// and a twiddle table that reaches W_N.
-typedef void (*RegRingKernel)(RingTable, int, JobList, const float2 *, int, float, const int *, const float2 *);
-static RegRingKernel pick_reg_kernel(const tl_plan *p, const FftGroup &g, int *lg) {
-  if (p->precision == TL_FP64 || !p->ring_reg || g.M != 0 || g.ni_min != g.ni_max) return nullptr;
-  const int N = 4 * g.ni_min;
-  if ((N & (N - 1)) != 0 || N <= p->mmax || N > p->tw_len) return nullptr;
-  // every ring of the group starts a 256-pixel tile of the derivative maps: north cap
-  // rings at 2 i (i - 1), south ones at Npix - 2 i (i + 1), belt rings at
-  // 2 N (N - 1) + k 4 N (N = nside)
-  const long long i = g.ni_min, ns = p->nside, T = kD3Tile;
-  const bool aligned = (i == ns) ? ((2 * ns * (ns - 1)) % T == 0 && (4 * ns) % T == 0)
-                                 : ((2 * i * (i - 1)) % T == 0 && (p->npix - 2 * i * (i + 1)) % T == 0);
-  if (!aligned) return nullptr;
-  *lg = 31 - __builtin_clz((unsigned)N);
-  switch (*lg) {
-    case 10: return ringfft_reg_kernel<10>;
-    case 11: return ringfft_reg_kernel<11>;
-    case 12: return ringfft_reg_kernel<12>;
-    case 13: return ringfft_reg_kernel<13>;
-    default: return nullptr;
-  }
 }
 
 template <typename T>
@@ -1114,28 +786,34 @@ static cudaError_t ringfft_t(const tl_plan *p, const void *const *planes, const 
     jl.job[i].out = jobs[i].out;
     jl.job[i].tile = jobs[i].tile;
   }
-  const int lgtw = 31 - __builtin_clz((unsigned)p->tw_len);
-  for (int gi = 0; gi < p->fft_ngroups; ++gi) {
-    const FftGroup &g = p->fft_groups[gi];
+  // single precision: the synthesis kernels take every ring that one of their grids fits, and
+  // the rest (belt and outer cap rings above Nside 2048) go the general way
+  const FftGroup *groups = p->fft_groups;
+  const int *rings = p->fft_rings;
+  int ngroups = p->fft_ngroups;
+  if (sizeof(T) == 4 && p->sy_ngroups > 0) {
+    // one plane's maps one after another, by increasing phi-derivative (the general kernel
+    // takes the jobs in the caller's pairs)
+    JobList by_plane = jl;
+    std::stable_sort(by_plane.job, by_plane.job + njobs, [](const JobDev &a, const JobDev &b) {
+      return a.in != b.in ? (uintptr_t)a.in < (uintptr_t)b.in : a.k < b.k;
+    });
+    TL_CUDA_TRY(launch_ring_synth(p, by_plane, s));
+    groups = p->rest_groups;
+    rings = p->rest_rings;
+    ngroups = p->rest_ngroups;
+  }
+  for (int gi = 0; gi < ngroups; ++gi) {
+    const FftGroup &g = groups[gi];
     dim3 grid(g.count, (njobs + 1) / 2);
-    int lg = 0;
-    const RegRingKernel rk = (sizeof(T) == 4) ? pick_reg_kernel(p, g, &lg) : nullptr;
-    if (rk) {
-      const size_t smem = sizeof(float2) * (size_t)((1 << lg) + (1 << (lg - 4)));
-      TL_CUDA_TRY(raise_smem((const void *)rk, smem));
-      rk<<<grid, 1 << (lg - 4), smem, s>>>(p->ring, p->mmax, jl, (const float2 *)p->twiddle, lgtw,
-                                           (float)(1.0 / (double)(p->lmax + 1)), p->fft_rings + g.first,
-                                           (const float2 *)p->phase);
-      continue;
-    }
-    const int batch = group_batch(p, g);
-    const RingKernel<T> kern = pick_ring_kernel<T>(p, g);
-    const int nt = group_threads(p, g);
-    TL_CUDA_TRY(raise_smem((const void *)kern, group_smem(p, g, batch, nt)));
-    kern<<<grid, nt, group_smem(p, g, batch, nt), s>>>(
-        p->ring, p->nside, p->mmax, jl, p->blue,
-        (const typename RealTraits<T>::T2 *)p->twiddle, p->tw_len, batch, (T)(1.0 / (double)(p->lmax + 1)),
-        p->fft_rings + g.first, (const typename RealTraits<T>::T2 *)p->phase);
+    const int batch = group_batch(p, g, false);
+    const auto kern = g.M ? ringfft_kernel<T, true> : ringfft_kernel<T, false>;
+    const size_t smem = group_smem(p, g, batch, false);
+    TL_CUDA_TRY(raise_smem((const void *)kern, smem));
+    kern<<<grid, 512, smem, s>>>(p->ring, p->nside, p->mmax, jl, p->blue,
+                                 (const typename RealTraits<T>::T2 *)p->twiddle, p->tw_len, batch,
+                                 (T)(1.0 / (double)(p->lmax + 1)), rings + g.first,
+                                 (const typename RealTraits<T>::T2 *)p->phase);
   }
   return cudaGetLastError();
 }
@@ -1168,12 +846,13 @@ static cudaError_t ringfft_adj_t(const tl_plan *p, void *const *planes, const Ad
     jl.job[i].nk = jobs[i].nk;
     jl.job[i].pad = 0;
   }
-  TL_CUDA_TRY(set_group_smem(p, ringfft_adj_kernel<T>));
   for (int gi = 0; gi < p->fft_ngroups; ++gi) {
     const FftGroup &g = p->fft_groups[gi];
-    const int batch = group_batch(p, g);
+    const int batch = group_batch(p, g, true);
+    const size_t smem = group_smem(p, g, batch, true);
     dim3 grid(g.count, njobs);
-    ringfft_adj_kernel<T><<<grid, 512, group_smem(p, g, batch, 512), s>>>(
+    TL_CUDA_TRY(raise_smem((const void *)ringfft_adj_kernel<T>, smem));
+    ringfft_adj_kernel<T><<<grid, 512, smem, s>>>(
         p->ring, p->mmax, p->npix, p->nmaps, jl, p->blue,
         (const typename RealTraits<T>::T2 *)p->twiddle, p->tw_len, batch, (double)(p->lmax + 1),
         p->fft_rings + g.first, (const typename RealTraits<T>::T2 *)p->phase, p->blue_reg_lg);

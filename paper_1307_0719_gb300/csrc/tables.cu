@@ -138,7 +138,8 @@ long long host_bluestein_layout(int nside, long long *off, int *ml, int *maxm) {
 // Rings of each ring-FFT launch: the equatorial belt, then the caps by Bluestein
 // length M (largest first), then the power-of-two caps; each group's rings are
 // ordered by decreasing length. No allocation.
-int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGroup *groups, int *order) {
+int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGroup *groups, int *order,
+                    const unsigned char *use) {
   int ng = 0, n = 0;
   auto key_of = [&](int r) {
     const int ni = nphi[r] / 4;
@@ -147,7 +148,7 @@ int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGr
   auto add = [&](int key) {
     const int first = n;
     for (int r = 0; r < nrings; ++r)
-      if (key_of(r) == key) order[n++] = r;
+      if ((!use || use[r]) && key_of(r) == key) order[n++] = r;
     if (n == first) return true;
     std::sort(order + first, order + n, [&](int a, int b) { return nphi[a] != nphi[b] ? nphi[a] > nphi[b] : a < b; });
     if (ng == TL_MAX_FFT_GROUPS) return false;
@@ -163,7 +164,46 @@ int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGr
   for (int M = 1 << 30; M >= 2; M >>= 1)
     if (M <= 4 * nside && !add(M)) return -1;
   if (!add(0)) return -1;
-  return n == nrings ? ng : -1;
+  int want = nrings;
+  if (use) {
+    want = 0;
+    for (int r = 0; r < nrings; ++r) want += use[r] != 0;
+  }
+  return n == want ? ng : -1;
+}
+
+// The Legendre stage holds a function of (l, m) at zero until it reaches 2^-32. Beyond the
+// turning point sin theta_t = m / L (L = lmax + 1/2) the largest l is damped by e^-S,
+//   S = int_theta^theta_t sqrt(m^2 / sin^2 t - L^2) dt
+//     = m artanh(R / (m cos theta)) - L artanh(R / (L cos theta)),  R^2 = m^2 - L^2 sin^2 theta
+// (the first-order WKB exponent; smaller l are damped more). Its prefactor is of order one:
+// S = 26 against 32 ln 2 = 22.2, and three more in m for the spin's shift, leave no ring of
+// any (Nside, lmax) tried with a non-zero coefficient beyond (spin 0 and 2; slack about 7).
+void host_ring_bands(int nside, int lmax, const double *sint, const double *z, int *mcut) {
+  const double L = lmax + 0.5;
+  const int nr = 4 * nside - 1;
+  for (int r = 0; r < 2 * nside; ++r) {
+    const double s = sint[r], c = fabs(z[r]);
+    auto damp = [&](int m) {
+      if (m <= L * s || c == 0.0) return 0.0;
+      const double R = sqrt(m * (double)m - L * L * s * s);
+      const double a = R / (m * c), b = R / (L * c);
+      if (a >= 1.0 || b >= 1.0) return 1e9;
+      return m * atanh(a) - L * atanh(b);
+    };
+    int lo = 0, hi = lmax;
+    if (damp(lmax) < 26.0) {
+      lo = lmax;
+    } else {
+      while (hi - lo > 1) {
+        const int k = (lo + hi) / 2;
+        if (damp(k) < 26.0) lo = k;
+        else hi = k;
+      }
+      lo = lo + 3 < lmax ? lo + 3 : lmax;
+    }
+    mcut[r] = mcut[nr - 1 - r] = lo;
+  }
 }
 
 // long enough for every Bluestein length and for a whole belt ring (4 nside), whose
