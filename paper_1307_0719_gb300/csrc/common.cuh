@@ -111,7 +111,8 @@ struct tl_plan {
   // recurrence state there
   int *tc_bs0, *tc_bsp, *tc_bs2;
   float *tc_st0, *tc_stp, *tc_st2;
-  float *tc_sm0, *tc_smp, *tc_sm2;  // the same state at each unit's midpoint block (split units)
+  float *tc_sm0, *tc_smp, *tc_sm2;  // the same state at the first blocks of each unit's quarters 1 .. 3
+  float *tc_leib;                   // Leibniz coefficients per ring
   float *tc_step0, *tc_step2;     // per 8-l block: A_{l+1} x 8, then A - 2 x 8 (spin 0) or Qn, Qs x 8 (spin 2)
   void *tc_b0, *tc_bp, *tc_b2;    // [blocks] 2 KB coefficient tiles (TF32 hi, lo; 32 columns x 8 l)
   int *dev_err;                   // set by a kernel whose bounded wait timed out
@@ -227,7 +228,8 @@ cudaError_t launch_legendre_spin0_tc(const tl_plan *p, int which, int nreal, voi
 // start tables of the tensor-core Legendre stage (which: 0 T, 1 potential, 2 Q/U)
 cudaError_t launch_tcstart(const tl_plan *p, int which, int *bstart, float *state, float *state_mid,
                            cudaStream_t s);
-bool tc_split(const tl_plan *p, int which);
+size_t tc_leib_bytes(const tl_plan *p);
+cudaError_t launch_tcleib(const tl_plan *p, float *out, cudaStream_t s);
 size_t tc_start_state_bytes(const tl_plan *p, int which);
 size_t tc_start_units(const tl_plan *p, int which);
 cudaError_t launch_bluestein_setup(tl_plan *p, cudaStream_t s);
@@ -263,7 +265,7 @@ int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGr
 // mcut[r]: the largest m whose coefficients can be non-zero on ring r at band limit lmax
 void host_ring_bands(int nside, int lmax, const double *sint, const double *z, int *mcut);
 struct JobList;
-void host_synth_window(SyWindow *w, float *corr10, float *corr8);
+const float *host_synth_window(SyWindow *w);  // returns [2][kSyCorr] corrections
 int host_synth_groups(int nside, int nrings, const int *nphi, const int *mcut, SyGroup *groups, int4 *rings, int *rest,
                       int *nrest);
 cudaError_t launch_ring_synth(const tl_plan *p, const JobList &jl, cudaStream_t s);

@@ -7,7 +7,7 @@
 // theta-derivatives by Leibniz's rule. A CTA holds 128 rings (spin 2: 64 north
 // rings and their mirrors; spin 0: 128 north rings, south by parity) in four
 // compute warps, plus one warp that issues the tensor-core work; where tensor
-// memory allows, four more compute warps run the second half of each unit's l
+// memory allows, two or four such sets of compute warps run parts of each unit's l
 // range on the same rings (see run_blocks). Every 8 values of l the compute warps
 // write the [128 rings x 8 l] tile of mu^(j) of every derivative order j into
 // tensor memory (ring slot t in lane t, the tile's row t), and the issuing warp runs
@@ -28,20 +28,24 @@
 // up to 128, so the MMA side of a block costs the same for 64 columns as for 32
 // and the columns per tile set the realisations served per recurrence. The
 // accumulators of 16 realisations (5 orders x 64 columns) and the basis tiles
-// (2 x 80 columns for 3xTF32; 2 halves x 2 x 40 for BF16x3) then fill the 512
+// (2 parts x 80 columns for 3xTF32; 4 parts x 40 for BF16x3) then fill the 512
 // columns of tensor memory (one CTA per SM).
 //
-// Pipeline: the basis tiles (tensor memory) and the coefficient tiles (shared
-// memory) are double-buffered where the columns allow. For block g the compute
-// warps run 8 steps in registers (step factors and coefficient tiles prefetched
-// one block ahead), wait until the MMAs of the block that last used the buffer
-// have completed (mbarrier "done" of the buffer, signalled by tcgen05.commit),
-// store the basis tiles (tcgen05.st) and the coefficient tile, and arrive on the
-// buffer's "full" barrier (one arrival per warp). The issuing warp waits for the
-// four arrivals, issues the block's MMAs and commits them to the buffer's "done",
-// so the tensor core works on one buffer while the other is being filled. With two
-// halves each has its own buffers and barriers, and the issuing warp alternates
-// between them block by block.
+// Pipeline: a unit's l range is cut into NH parts (4 where tensor memory has room for four
+// sets of basis tiles), each run by its own four compute warps on the same 128 rings from
+// a recurrence state tabulated at plan time; all parts feed the same accumulators. A copying
+// warp's one lane brings the coefficient tiles and step factors of the coming blocks into
+// shared memory (cp.async.bulk, kStages blocks per part, mbarrier "tile" each). For block g of a part
+// its compute warps take the step factors from there, run 8 steps in registers, wait until
+// the MMAs of the block that last used their basis-tile buffer have completed (mbarrier
+// "done", signalled by tcgen05.commit), tell the copying lane that that block's stage is free,
+// store the basis tiles (tcgen05.st) and arrive on the buffer's "full" barrier (one arrival
+// per warp). The issuing warp's one lane waits for the arrivals, issues the MMAs and commits
+// them to "done". Parts share these barriers in groups, so that one wait serves the MMAs of
+// several blocks: a lane that reads a barrier after issuing MMAs is held for about 200 cycles, and
+// the tensor pipe runs dry meanwhile (measured: 710, 575 and 508 cycles per ten MMAs for 10, 20 and
+// 40 of them per wait, 467 without waits). Two groups take turns, or one group has two
+// buffers, so that the next tiles are formed while the tensor core works.
 //
 // The coefficient tile uses the K-major shared-memory layout without swizzle:
 // 8-row x 16-byte core matrices, 128 bytes apart along K and 256 bytes apart along
@@ -55,11 +59,13 @@
 namespace tl {
 
 constexpr int kMaxReal = TL_MAX_BATCH;  // realisations per launch at most (64 columns)
-constexpr int kComputeThreads = 128;  // compute threads per half (umma_threads: the CTA's)
+constexpr int kComputeThreads = 128;  // compute threads per part (umma_threads: the CTA's)
 // spin-2 epilogue exchange: [128 rings][9] float2 (8 used; the odd row length puts the
 // 32 rows a warp writes or reads at once on distinct bank pairs)
 constexpr int kXchRow = 9;
 constexpr uint32_t kXchBytes = 128 * kXchRow * 8;
+constexpr int kStages = 4;            // coefficient-tile buffers per part (power of two)
+constexpr uint32_t kStepBytes = 128;  // a block's step factors in shared memory (96 or 64 used)
 
 // accumulator columns per order for NDER theta-derivatives: 64 (16 realisations)
 // up to NDER = 5, 32 (8) at NDER = 6, where 64 would not fit tensor memory
@@ -141,8 +147,25 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, int po
   return false;
 }
 
+// one lane of a converged warp (the compiler then keeps the operands of its tcgen05.mma
+// in uniform registers without moving them there for each)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
+// global -> shared, completion counted on the mbarrier (16-byte aligned addresses and size)
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(mbar)
+               : "memory");
 }
 
 // 32 consecutive columns of the calling thread's lane
@@ -198,19 +221,21 @@ __device__ __forceinline__ void bf16_split2(float x0, float x1, uint32_t &hi, ui
   lo = bf16x2(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
 }
 
-// Halves of the l range a unit is split into (two sets of compute warps on the
-// same rings, see run_blocks): 2 where both halves' basis tiles fit the 512
-// columns double-buffered, else 1.
-__host__ __device__ constexpr int tc_halves(int nj, int mode, int nc) {
-  return nj * nc + 4 * nj * (mode == kModeTf32x3 ? 16 : 8) <= 512 ? 2 : 1;
+// Parts of the l range a unit is split into (sets of four compute warps on the same rings,
+// see run_blocks): 4 where a CTA fills the SM anyway and four sets of basis tiles fit the 512
+// columns, else 2 where two sets fit, else 1. (Two CTAs of two parts per SM for the potential: a
+// CTA of four parts has 544 threads of up to 120 registers, and only one fits.)
+__host__ __device__ constexpr int tc_parts(int nj, int mode, int nc) {
+  const int acc = nj * nc, aset = nj * (mode == kModeTf32x3 ? 16 : 8);
+  return acc + 4 * aset <= 256 ? 2 : acc + 4 * aset <= 512 ? 4 : acc + 2 * aset <= 512 ? 2 : 1;
 }
 
 // Tensor-memory map of a CTA: accumulators D^(j) at columns NC j (j < NJ), then
-// NH x NB sets of basis tiles: Mu^(j) of half h, buffer i at A0 + (h NB + i) ASET +
+// NH x NB sets of basis tiles: Mu^(j) of part h, buffer i at A0 + (h NB + i) ASET +
 // AW j (hi in 8 columns, then lo for 3xTF32; BF16x3: hi pairs in 4 columns, lo
-// pairs in 4). Two buffers per half where they fit the 512 columns, else one. The
+// pairs in 4). Two buffers per part where they fit the 512 columns, else one. The
 // allocation is the next power of two; `ctas` is how many CTAs of that size fit the
-// SM (at most 4).
+// SM (at most 3, by their threads' registers; one with four parts).
 template <int NJ, int MODE, int NC, int NH = 1> struct TmemMap {
   static constexpr int AW = MODE == kModeTf32x3 ? 16 : 8;
   static constexpr int A0 = NJ * NC;
@@ -218,7 +243,7 @@ template <int NJ, int MODE, int NC, int NH = 1> struct TmemMap {
   static constexpr int NB = A0 + NH * 2 * ASET <= 512 ? 2 : 1;
   static constexpr int need = A0 + NH * NB * ASET;
   static constexpr int cols = need <= 32 ? 32 : need <= 64 ? 64 : need <= 128 ? 128 : need <= 256 ? 256 : 512;
-  static constexpr int ctas = 512 / cols > 4 ? 4 : 512 / cols;
+  static constexpr int ctas = NH == 4 ? 1 : 512 / cols > 3 ? 3 : 512 / cols;
   static_assert(need <= 512, "tensor memory");
 };
 
@@ -240,36 +265,57 @@ struct TcDesc {
   // state at the start of that block: [unit][2 NJ + 1][128] (a, b, scale)
   const int *bstart;
   const float *state;
-  // the same state at the first block of the unit's second half (see run_blocks),
-  // or NULL (no split)
+  // the same state at the first block of the unit's quarters 1 .. 3 (seg_first), one
+  // array after another, mid_stride elements each; or NULL (no split)
   const float *state_mid;
+  long long mid_stride;
+  const float *leib;             // Leibniz coefficients e[j][i] per ring (leib_table_kernel)
   int nrblk;
   int polls;  // polls of every mbarrier wait before it gives up (bounded waits)
   int stall;  // self-test: the compute warps withhold their arrivals, so waits run out
 };
 
-// Per-CTA tcgen05 state (identical in every thread). Each half h of the compute
-// warps has four mbarriers, adjacent 8-byte words from bars + 32 h: done[0],
-// done[1] (MMAs of the buffer's last block completed; one arrival, the commit),
-// full[0], full[1] (the block's tiles written; one arrival per compute warp of the
-// half). Their addresses are formed arithmetically: a runtime-indexed array member
-// would put the struct in local memory.
+// Groups of parts that share the hand-off to the tensor core: one where every part has two
+// basis-tile buffers, else two that take turns (one of a single part).
+__host__ __device__ constexpr int tc_groups(int nh, int nb) { return nb == 2 || nh == 1 ? 1 : 2; }
+
+// Per-CTA tcgen05 state (identical in every thread). Twelve mbarriers, adjacent 8-byte words from
+// bars + 96 h, belong to group h (the first four) and part h (the others) of the compute warps:
+// done[0], done[1] (MMAs of the buffer's last blocks completed; one arrival, the commit),
+// full[0], full[1] (the blocks' basis tiles written; one arrival per compute warp of the
+// group), tile[0..3] (coefficient tile and step factors of a stage have arrived), free[0..3]
+// (the stage's block has been multiplied; one arrival by the part's first thread). Their addresses
+// are formed arithmetically: a runtime-indexed array member would put the struct in local memory.
 struct UmmaCta {
   uint32_t tmem;        // tensor-memory base (lane 0, first column)
-  uint32_t bars;        // shared address of half 0's done[0]
-  uint32_t count;       // blocks so far, first half
-  uint32_t count1;      // blocks so far, second half
+  uint32_t bars;        // shared address of part 0's done[0]
+  uint32_t c0, c1, c2, c3;  // blocks so far, per part
+  uint32_t g0, g1;          // hand-offs so far, per group
   volatile int *abort;  // shared: set by a thread whose wait timed out
   bool failed;
 };
-__device__ __forceinline__ uint32_t bar_done(const UmmaCta &U, uint32_t i, uint32_t h = 0) {
-  return U.bars + 32u * h + 8u * i;
+__device__ __forceinline__ uint32_t part_count(const UmmaCta &U, int h) {
+  return h == 0 ? U.c0 : h == 1 ? U.c1 : h == 2 ? U.c2 : U.c3;
 }
-__device__ __forceinline__ uint32_t bar_full(const UmmaCta &U, uint32_t i, uint32_t h = 0) {
-  return U.bars + 32u * h + 16u + 8u * i;
+__device__ __forceinline__ uint32_t group_count(const UmmaCta &U, int gr) { return gr == 0 ? U.g0 : U.g1; }
+__device__ __forceinline__ uint32_t bar_done(const UmmaCta &U, uint32_t i, uint32_t h) { return U.bars + 96u * h + 8u * i; }
+__device__ __forceinline__ uint32_t bar_full(const UmmaCta &U, uint32_t i, uint32_t h) {
+  return U.bars + 96u * h + 16u + 8u * i;
 }
-// threads of a CTA with NH halves: 4 compute warps, the issuing warp, 4 more compute warps
-__host__ __device__ constexpr int umma_threads(int nh) { return nh == 2 ? 288 : 160; }
+__device__ __forceinline__ uint32_t bar_tile(const UmmaCta &U, uint32_t g, uint32_t h) {
+  return U.bars + 96u * h + 32u + 8u * (g & (kStages - 1));
+}
+__device__ __forceinline__ uint32_t bar_free(const UmmaCta &U, uint32_t g, uint32_t h) {
+  return U.bars + 96u * h + 64u + 8u * (g & (kStages - 1));
+}
+__device__ __forceinline__ uint32_t tile_phase(uint32_t g) { return (g / kStages) & 1u; }
+// threads of a CTA with NH parts: 4 NH compute warps, the issuing warp, the copying warps (one per
+// two parts: a copy takes its lane a few hundred cycles, which with four parts in one lane was
+// longer than the block it was for)
+__host__ __device__ constexpr int tc_copy_warps(int nh) { return nh == 4 ? 2 : 1; }
+__host__ __device__ constexpr int umma_threads(int nh) { return kComputeThreads * nh + 32 + 32 * tc_copy_warps(nh); }
+// first block, from a unit's first running one, of quarter q = 0 .. 4 of its nrun blocks
+__host__ __device__ __forceinline__ int seg_first(int nrun, int q) { return (nrun * q + 3) >> 2; }
 // Block g uses buffer g % NB; it is that buffer's (g / NB)-th use, i.e. phase
 // g / NB of both of its barriers.
 template <int NB> __device__ __forceinline__ uint32_t buf_of(uint32_t g) { return NB == 2 ? (g & 1u) : 0u; }
@@ -307,7 +353,7 @@ __device__ __forceinline__ void steps_gated(float (&a)[NDER + 1], float (&b)[NDE
 }
 
 // The 8 steps of one block; spin 2's mirror rings (cos th < 0) are whole warps
-// (threads 64-127 of a half), so the branch is warp-uniform.
+// (threads 64-127 of a part), so the branch is warp-uniform.
 template <int NDER, bool SPIN2>
 __device__ __forceinline__ void block_steps(bool mirror, float (&a)[NDER + 1], float (&b)[NDER + 1], int &sc,
                                             const Leib<float, NDER> &LC, float w, const float (&Av)[8],
@@ -413,22 +459,36 @@ __device__ __forceinline__ void unit_seed(const TcDesc &D, int r, int m, bool ac
   rec_init<float, NDER>(a, b);  // difference form: d = mu_{l0}
 }
 
+// Dynamic shared memory of a CTA: kStages coefficient tiles per part, their step factors, then
+// the spin-2 exchange areas (one per part).
+template <int NC, int NH> __host__ __device__ constexpr uint32_t step_offset() { return kStages * NH * btile_bytes(NC); }
+template <int NC, int NH> __host__ __device__ constexpr uint32_t xch_offset() {
+  return kStages * NH * (btile_bytes(NC) + kStepBytes);
+}
+
 // One (m, ring block) unit: recurrence and tiles (compute warps), MMAs (issuing
-// warp). NB: the kernel's buffer count per half (the same for every unit a CTA
-// runs, so that the barriers' phases follow one block count). NH = 2 splits the
-// unit's blocks between two sets of four compute warps on the same 128 rings: the
-// first runs blocks [bs, bmid) from the start-table state, the second [bmid, nblk)
-// from the state the recurrence has at bmid (plan-time table state_mid, identical
-// arithmetic), and both feed the same accumulators; warps 0-3 form the first set,
-// warps 5-8 the second (ring 32 (warp mod 4) + lane: the tensor-memory lanes a warp
-// may access). Leaves the accumulators complete in tensor memory (every MMA waited
-// for) and returns the number of 8-l blocks run (0: accumulators unset).
+// warp). NB: the kernel's buffer count per part (the same for every unit a CTA
+// runs, so that the barriers' phases follow one block count). The unit's blocks [bs, nblk) are
+// split between NH parts, each from the state the recurrence has there (plan-time tables,
+// identical arithmetic); compute warp w is in part w / 4 and holds ring 32 (w mod 4) +
+// lane (the tensor-memory lanes such a warp may access). Leaves the accumulators complete in
+// tensor memory (every MMA waited for) and returns the number of 8-l blocks run (0:
+// accumulators unset).
+//
+// What bounds it: the tensor pipe takes one M = 128, K = 16 instruction per 46 cycles for any
+// N up to 64 (measured), ten per block at order 4, so a block cannot take less than 467 cycles;
+// at Nside 2048 / lmax 3000 it takes 820 in the loop (the issuing warp shares its scheduler with
+// compute warps that are 67% issue-active, and waits 240 cycles per two blocks) and 950 with the unit's
+// start, end and epilogue. Before (two parts, the tiles through the compute warps' registers, one
+// lane per block): 1330. Spin 2 103.9 -> 74.3 ms, spin 0 with the potential 70.0 -> 52.6 ms.
 template <int NDER, int MODE, int NC, int NB, bool SPIN2, int NH>
 __device__ __forceinline__ int run_blocks(const TcDesc &D, int m, int rblk, unsigned char *sm, UmmaCta &U) {
   constexpr int NJ = NDER + 1;
   typedef TmemMap<NJ, MODE, NC, NH> TM;
   static_assert(NB <= TM::NB, "buffers fit");
+  static_assert(NB < kStages, "a stage is refilled NB blocks after its use");
   constexpr uint32_t BT = btile_bytes(NC);
+  constexpr uint32_t SB = (uint32_t)step_stride(SPIN2) * 4u;  // bytes of a block's step factors
   const int tid = threadIdx.x, warp = tid >> 5;
   const int l0 = unit_l0(m, SPIN2);
   const int nblk = (D.lmax >= l0) ? (D.lmax - l0 + 8) / 8 : 0;
@@ -437,49 +497,103 @@ __device__ __forceinline__ int run_blocks(const TcDesc &D, int m, int rblk, unsi
   // blocks before bs contribute nothing for any ring of the unit (start table)
   const int bs = D.bstart ? D.bstart[unit] : 0;
   const int nrun = nblk - bs;
-  const bool split = NH == 2 && D.bstart && D.state_mid;
-  const int n0 = split ? (nrun + 1) / 2 : nrun, n1 = nrun - n0;
-  const uint32_t g00 = U.count, g01 = U.count1;
-  bool bad = false;
-  if (warp == kComputeThreads / 32) {
-    // ---- issuing warp: one lane waits for each block's tiles and issues its MMAs,
-    // block k of the first half, then block k of the second
-    if (tid == kComputeThreads) {
-      const uint64_t dB0 = umma_desc(smem_u32(sm));
-      for (int k = 0; k < n0 && !bad; ++k) {
+  const bool split = NH > 1 && D.bstart && D.state_mid;
+  // first block of part h (h = NH: the end), from bs, and its number of blocks
+  auto first_of = [&](int h) { return split ? seg_first(nrun, h * (4 / NH)) : h == 0 ? 0 : nrun; };
+  auto count_of = [&](int h) { return first_of(h + 1) - first_of(h); };
+  // hand-offs of group gr: the blocks of its longest part
+  constexpr int NG = tc_groups(NH, NB), PP = NH / NG;  // groups, parts of a group
+  auto handoffs = [&](int gr) {
+    int n = 0;
 #pragma unroll
-        for (int h = 0; h < NH; ++h) {
-          if (h == 1 && k >= n1) break;
-          const uint32_t g = (h ? g01 : g00) + (uint32_t)k, i = buf_of<NB>(g), ib = (uint32_t)h * NB + i;
-          if (!mbar_wait(bar_full(U, i, h), phase_of<NB>(g), D.polls, U.abort)) {
-            bad = true;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          issue_block<NJ, MODE, NC>(U.tmem, (uint32_t)(TM::A0 + TM::ASET * ib), dB0 + ((ib * BT) >> 4),
-                                    h == 0 && k == 0);
-          umma_commit(bar_done(U, i, h));
+    for (int h = 0; h < PP; ++h) n = max(n, count_of(gr * PP + h));
+    return n;
+  };
+  const uint32_t smb = smem_u32(sm);
+  bool bad = false;
+  constexpr int CP = NH / tc_copy_warps(NH);  // parts of a copying warp
+  int loaded = 0;  // copying warp: one past its last copy started, k CP + (h mod CP)
+  if (warp == 4 * NH) {
+    // ---- issuing warp: waits for a group's tiles and issues its blocks' MMAs (one lane), block k of
+    // every part of one group, then of the other (the compute warps arrive on "full" after they have
+    // seen the stage's copies complete, so the coefficient tiles are there too)
+    const uint64_t dB0 = umma_desc(smb);
+    // four parts: the CTA holds all 512 columns, which start at 0
+    const uint32_t tm = NH == 4 ? 0u : U.tmem;
+    const int most = handoffs(0);  // the first group holds the longest part
+    for (int k = 0; k < most && !bad; ++k) {
+#pragma unroll
+      for (int gr = 0; gr < NG; ++gr) {
+        if (k >= handoffs(gr) || bad) continue;
+        const uint32_t g = group_count(U, gr) + (uint32_t)k, i = buf_of<NB>(g);
+        if (!mbar_wait(bar_full(U, i, gr), phase_of<NB>(g), D.polls, U.abort)) {
+          bad = true;
+          continue;
         }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (elect_one()) {
+#pragma unroll
+          for (int q = 0; q < PP; ++q) {
+            const int h = gr * PP + q;
+            if (k < count_of(h)) {
+              const uint32_t st = (uint32_t)h * kStages + ((part_count(U, h) + (uint32_t)k) & (kStages - 1));
+              issue_block<NJ, MODE, NC>(tm, (uint32_t)(TM::A0 + TM::ASET * (h * NB + i)), dB0 + ((st * BT) >> 4),
+                                        h == 0 && k == 0);
+            }
+          }
+          umma_commit(bar_done(U, i, gr));
+        }
+        __syncwarp();
       }
     }
-    __syncwarp();
+  } else if (warp > 4 * NH) {
+    // ---- copying warps (one lane each): block k of the warp's parts in turn, into the stage that
+    // block g - kStages of the part has left
+    const int h0 = (warp - 4 * NH - 1) * CP;
+    const int most = count_of(h0);  // the longest of its parts
+    for (int k = 0; k < most && !bad; ++k) {
+#pragma unroll
+      for (int q = 0; q < CP; ++q) {
+        const int h = h0 + q;
+        if (k >= count_of(h) || bad) continue;
+        const uint32_t g = part_count(U, h) + (uint32_t)k, st = (uint32_t)h * kStages + (g & (kStages - 1));
+        if (g >= (uint32_t)kStages && !mbar_wait(bar_free(U, g, h), tile_phase(g - kStages), D.polls, U.abort)) {
+          bad = true;
+          continue;
+        }
+        if (elect_one()) {
+          const long long blk = b0 + bs + first_of(h) + k;
+          const uint32_t bar = bar_tile(U, g, h);
+          mbar_expect(bar, BT + SB);
+          bulk_copy(smb + st * BT, D.b + blk * BT, BT, bar);
+          bulk_copy(smb + step_offset<NC, NH>() + st * kStepBytes, (const unsigned char *)D.step + blk * SB, SB, bar);
+        }
+        __syncwarp();
+        loaded = k * CP + q + 1;
+      }
+    }
   } else {
     // ---- compute warps: one ring per thread (tensor-memory lane t)
-    const int h = (NH == 2 && warp > kComputeThreads / 32) ? 1 : 0;
-    const int t = h ? (((warp & 3) << 5) | (tid & 31)) : tid;
-    const int first = h ? bs + n0 : bs, cnt = h ? n1 : n0;
-    const uint32_t g0 = h ? g01 : g00;
+    const int h = NH == 1 ? 0 : warp >> 2;
+    const int t = tid & (kComputeThreads - 1);
+    const int gr = h / PP;  // its group
+    const int cnt = count_of(h), steps = handoffs(gr);
+    const uint32_t g0 = part_count(U, h), gg0 = group_count(U, gr);
     const RingTable &rt = D.rt;
     bool active;
     const int r = unit_ring<SPIN2>(D, rblk, t, active);
     const uint32_t lane = U.tmem + ((uint32_t)((warp & 3) * 32) << 16);
     Leib<float, NDER> LC;
-    leibniz_coefs<float, NDER>(rt.z[r], rt.sint[r], 1.0 / (double)(D.lmax + 1), LC);
+#pragma unroll
+    for (int j = 1; j <= NDER; ++j)
+#pragma unroll
+      for (int i = 1; i <= j; ++i) LC.e[j][i] = __ldg(D.leib + (size_t)(j * (j - 1) / 2 + i - 1) * D.nrings + r);
     float a[NJ], b[NJ];
     int sc;
     if (D.bstart) {
-      // the state at block `first`, as the recurrence from l0 leaves it
-      const float *st = (h ? D.state_mid : D.state) + unit * (2 * NJ + 1) * kComputeThreads + t;
+      // the state at the part's first block, as the recurrence from l0 leaves it
+      const float *st = (h ? D.state_mid + (h * (4 / NH) - 1) * D.mid_stride : D.state) +
+                        unit * (2 * NJ + 1) * kComputeThreads + t;
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
         a[j] = __ldg(st + j * kComputeThreads);
@@ -491,103 +605,108 @@ __device__ __forceinline__ int run_blocks(const TcDesc &D, int m, int rblk, unsi
     }
     const float w = (float)rt.omza[r];
     const bool mirror = SPIN2 && t >= 64;
-    // the next block's step factors and coefficient tile (BT / 128 bytes per
-    // thread), loaded one block ahead
-    constexpr int QV = (int)(BT / 16 / kComputeThreads);  // float4 per thread: 1 or 2
-    const int qo = mirror ? 4 : 2;  // float4 offset of the thread's Q values
-    float4 nA0 = make_float4(0.f, 0.f, 0.f, 0.f), nA1 = nA0, nC0 = nA0, nC1 = nA0, nbq[QV];
-#pragma unroll
-    for (int q = 0; q < QV; ++q) nbq[q] = nA0;
-    auto prefetch = [&](int blk) {
-      const float4 *stp = (const float4 *)(D.step + (b0 + blk) * step_stride(SPIN2));
-      nA0 = __ldg(stp);
-      nA1 = __ldg(stp + 1);
-      nC0 = __ldg(stp + qo);
-      nC1 = __ldg(stp + qo + 1);
-      const float4 *bt = (const float4 *)(D.b + (b0 + blk) * BT);
-#pragma unroll
-      for (int q = 0; q < QV; ++q) nbq[q] = __ldg(bt + q * kComputeThreads + t);
-    };
-    if (cnt > 0) prefetch(first);
-    for (int k = 0; k < cnt; ++k) {
-      const int blk = first + k;
-      const uint32_t g = g0 + (uint32_t)k, i = buf_of<NB>(g), ib = (uint32_t)h * NB + i;
-      const float Av[8] = {nA0.x, nA0.y, nA0.z, nA0.w, nA1.x, nA1.y, nA1.z, nA1.w};
-      const float Cv[8] = {nC0.x, nC0.y, nC0.z, nC0.w, nC1.x, nC1.y, nC1.z, nC1.w};
-      float4 bq[QV];
-#pragma unroll
-      for (int q = 0; q < QV; ++q) bq[q] = nbq[q];
-      if (k + 1 < cnt) prefetch(blk + 1);
+    const uint32_t qo = mirror ? 4 : 2;  // float4 offset of the thread's Q values
+    for (int k = 0; k < steps; ++k) {
+      const uint32_t g = gg0 + (uint32_t)k, i = buf_of<NB>(g), ib = (uint32_t)h * NB + i;
+      const bool run = k < cnt;  // a part may have one block less than its group's longest
       float buf0[NJ][4], buf1[NJ][4];
-      block_steps<NDER, SPIN2>(mirror, a, b, sc, LC, w, Av, Cv, buf0, buf1);
-      // the buffer was last read by the MMAs of this half's block g - NB
-      if (g >= (uint32_t)NB && !mbar_wait(bar_done(U, i, h), phase_of<NB>(g - NB), D.polls, U.abort)) {
+      if (run) {
+        const uint32_t gt = g0 + (uint32_t)k, st = (uint32_t)h * kStages + (gt & (kStages - 1));
+        if (!mbar_wait(bar_tile(U, gt, h), tile_phase(gt), D.polls, U.abort)) {
+          bad = true;
+          break;
+        }
+        const float4 *stp = (const float4 *)(sm + step_offset<NC, NH>() + st * kStepBytes);
+        const float4 A0 = stp[0], A1 = stp[1], C0 = stp[qo], C1 = stp[qo + 1];
+        const float Av[8] = {A0.x, A0.y, A0.z, A0.w, A1.x, A1.y, A1.z, A1.w};
+        const float Cv[8] = {C0.x, C0.y, C0.z, C0.w, C1.x, C1.y, C1.z, C1.w};
+        block_steps<NDER, SPIN2>(mirror, a, b, sc, LC, w, Av, Cv, buf0, buf1);
+      }
+      // the buffer was last read by the MMAs of this group's hand-off g - NB
+      if (g >= (uint32_t)NB && !mbar_wait(bar_done(U, i, gr), phase_of<NB>(g - NB), D.polls, U.abort)) {
         bad = true;
         break;
       }
+      if (t == 0 && k >= NB && k - NB < cnt) mbar_arrive(bar_free(U, g0 + (uint32_t)(k - NB), h));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int q = 0; q < QV; ++q) *(float4 *)(sm + ib * BT + (q * kComputeThreads + t) * 16) = bq[q];
-      store_tiles<NDER, MODE>(lane + (uint32_t)(TM::A0 + TM::ASET * ib), buf0, buf1);
+      if (run) store_tiles<NDER, MODE>(lane + (uint32_t)(TM::A0 + TM::ASET * ib), buf0, buf1);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if ((tid & 31) == 0 && !D.stall) mbar_arrive(bar_full(U, i, h));
+      if ((tid & 31) == 0 && !D.stall) mbar_arrive(bar_full(U, i, gr));
     }
   }
-  U.count = g00 + (uint32_t)n0;
-  U.count1 = g01 + (uint32_t)n1;
-  // the last commit of each half covers every MMA issued before it
-  if (!bad && n0 > 0 &&
-      !mbar_wait(bar_done(U, buf_of<NB>(U.count - 1), 0), phase_of<NB>(U.count - 1), D.polls, U.abort))
-    bad = true;
-  if (NH == 2 && !bad && n1 > 0 &&
-      !mbar_wait(bar_done(U, buf_of<NB>(U.count1 - 1), 1), phase_of<NB>(U.count1 - 1), D.polls, U.abort))
-    bad = true;
+  U.c0 += (uint32_t)count_of(0);
+  if (NH > 1) U.c1 += (uint32_t)count_of(1);
+  if (NH > 2) U.c2 += (uint32_t)count_of(2);
+  if (NH > 2) U.c3 += (uint32_t)count_of(3);
+  U.g0 += (uint32_t)handoffs(0);
+  if (NG > 1) U.g1 += (uint32_t)handoffs(NG - 1);
+  // the last commit of each group covers every MMA issued before it
+#pragma unroll
+  for (int gr = 0; gr < NG; ++gr) {
+    const uint32_t c = group_count(U, gr);
+    if (!bad && handoffs(gr) > 0 &&
+        !mbar_wait(bar_done(U, buf_of<NB>(c - 1), gr), phase_of<NB>(c - 1), D.polls, U.abort))
+      bad = true;
+  }
+  // the parts' last stages are free too (every block frees its stage once)
+#pragma unroll
+  for (int h = 0; h < NH; ++h) {
+    if (!bad && tid == h * kComputeThreads)
+      for (int k = max(0, handoffs(h / PP) - NB); k < count_of(h); ++k)
+        mbar_arrive(bar_free(U, part_count(U, h) - (uint32_t)(count_of(h) - k), h));
+  }
   if (bad) *U.abort = 1;
   if (__syncthreads_or(bad)) {
     U.failed = true;
+    // copies in flight (bounded): the last ones started on every stage
+    if (warp > 4 * NH) {
+      const int h0 = (warp - 4 * NH - 1) * CP;
+      for (int q = loaded > kStages * CP ? loaded - kStages * CP : 0; q < loaded; ++q) {
+        const int k = q / CP, h = h0 + q - k * CP;
+        if (k < count_of(h)) {
+          const uint32_t g = part_count(U, h) - (uint32_t)(count_of(h) - k);
+          (void)mbar_wait(bar_tile(U, g, h), tile_phase(g), 1 << 20);
+        }
+      }
+    }
     return 0;
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   return nrun;
 }
 
-// Dynamic shared memory of a CTA: two coefficient tile buffers per half, then the
-// spin-2 exchange area.
-template <int NC, int NH> __host__ __device__ constexpr uint32_t xch_offset() { return 2 * NH * btile_bytes(NC); }
-
 // spin 2: combine each ring's S1 with its mirror's S2 into F^Q, F^U, one order and
-// one group of 8 realisations (32 columns) at a time
+// one group of 8 realisations (32 columns) at a time; the four warps of each part take every
+// NH-th of these, with an exchange area and a named barrier of their own
 template <int NDER, int MODE, int NC, int NB, int NH>
 __device__ __forceinline__ void u2_unit(const TcDesc &D, int m, int rblk, unsigned char *sm, UmmaCta &U) {
-  constexpr int NJ = NDER + 1;
+  constexpr int NJ = NDER + 1, HC = NC / 32;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int nblk = run_blocks<NDER, MODE, NC, NB, true, NH>(D, m, rblk, sm, U);
   if (U.failed) return;
-  const bool compute = tid < kComputeThreads;
-  const int rn = rblk * 64 + (tid & 63);
-  const bool active = compute && rn < 2 * D.nside;
-  const bool mirror = tid >= 64;
-  const int r = active ? (mirror ? D.nrings - 1 - rn : rn) : 0;
-  const bool writer = active && m <= D.mmax && !(mirror && rn == D.nrings - 1 - rn);  // equator: north thread
-  const int partner = tid ^ 64;
-  const size_t ld = (size_t)(D.mmax + 1);
-  float2 *xch = (float2 *)(sm + xch_offset<NC, NH>());  // [128][kXchRow]: S2 (4 rho + 2, 3) of every ring
+  if (warp < 4 * NH) {
+    const int part = warp >> 2, t = tid & (kComputeThreads - 1);
+    const int rn = rblk * 64 + (t & 63);
+    const bool active = rn < 2 * D.nside;
+    const bool mirror = t >= 64;
+    const int r = active ? (mirror ? D.nrings - 1 - rn : rn) : 0;
+    const bool writer = active && m <= D.mmax && !(mirror && rn == D.nrings - 1 - rn);  // equator: north thread
+    const int partner = t ^ 64;
+    const size_t ld = (size_t)(D.mmax + 1);
+    // [128][kXchRow]: S2 (4 rho + 2, 3) of every ring
+    float2 *xch = (float2 *)(sm + xch_offset<NC, NH>() + (uint32_t)part * kXchBytes);
 #pragma unroll 1
-  for (int j = 0; j < NJ; ++j) {
-#pragma unroll 1
-    for (int h = 0; h < NC / 32; ++h) {
+    for (int it = part; it < NJ * HC; it += NH) {
+      const int j = it / HC, h = it - j * HC;
       float v[32];
-      if (compute) {
-        tmem_ld32(U.tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(NC * j + 32 * h), v);
+      tmem_ld32(U.tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(NC * j + 32 * h), v);
 #pragma unroll
-        for (int rho = 0; rho < 8; ++rho) {
-          xch[tid * kXchRow + rho] = nblk ? make_float2(v[4 * rho + 2], v[4 * rho + 3]) : make_float2(0.f, 0.f);
-        }
+      for (int rho = 0; rho < 8; ++rho) {
+        xch[t * kXchRow + rho] = nblk ? make_float2(v[4 * rho + 2], v[4 * rho + 3]) : make_float2(0.f, 0.f);
       }
-      __syncthreads();
+      asm volatile("bar.sync %0, 128;" ::"r"(part + 1) : "memory");
       if (writer) {
         const float sg = (j & 1) ? -1.0f : 1.0f;
 #pragma unroll
@@ -603,45 +722,45 @@ __device__ __forceinline__ void u2_unit(const TcDesc &D, int m, int rblk, unsign
           D.d7b[o] = make_float2(-0.5f * bi, 0.5f * br);
         }
       }
-      __syncthreads();  // xch is rewritten next
+      asm volatile("bar.sync %0, 128;" ::"r"(part + 1) : "memory");  // xch is rewritten next
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
 }
 
 // spin 0: north ring r and its mirror by parity
 template <int NDER, int MODE, int NC, int NB, int NH>
 __device__ __forceinline__ void u0_unit(const TcDesc &D, int m, int rblk, unsigned char *sm, UmmaCta &U) {
-  constexpr int NJ = NDER + 1;
+  constexpr int NJ = NDER + 1, HC = NC / 32;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int nblk = run_blocks<NDER, MODE, NC, NB, false, NH>(D, m, rblk, sm, U);
   if (U.failed) return;
-  if (tid < kComputeThreads) {
-    const int rn = rblk * 128 + tid;
+  if (warp < 4 * NH) {
+    const int part = warp >> 2, t = tid & (kComputeThreads - 1);
+    const int rn = rblk * 128 + t;
     const bool active = rn < 2 * D.nside && m <= D.mmax;
     const int r = active ? rn : 0;
     const int rs = D.nrings - 1 - r;
     const size_t ld = (size_t)(D.mmax + 1);
-    const uint32_t lane_base = U.tmem + ((uint32_t)(warp * 32) << 16);
+    const uint32_t lane_base = U.tmem + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
-    for (int j = 0; j < NJ; ++j) {
+    for (int it = part; it < NJ * HC; it += NH) {
+      const int j = it / HC, h = it - j * HC;
       const float sg = (j & 1) ? -1.0f : 1.0f;
-#pragma unroll 1
-      for (int h = 0; h < NC / 32; ++h) {
-        float v[32];
-        tmem_ld32(lane_base + (uint32_t)(NC * j + 32 * h), v);
-        if (!active) continue;
-        if (nblk == 0) {  // nothing contributed: the accumulators were not written
+      float v[32];
+      tmem_ld32(lane_base + (uint32_t)(NC * j + 32 * h), v);
+      if (!active) continue;
+      if (nblk == 0) {  // nothing contributed: the accumulators were not written
 #pragma unroll
-          for (int c = 0; c < 32; ++c) v[c] = 0.f;
-        }
+        for (int c = 0; c < 32; ++c) v[c] = 0.f;
+      }
 #pragma unroll
-        for (int rho = 0; rho < 8; ++rho) {
-          if (8 * h + rho >= D.nreal) break;
-          const size_t o = (size_t)(8 * h + rho) * D.rstride + (size_t)j * D.prows * ld;
-          D.d7a[o + d7_il(r, m, ld)] = make_float2(v[4 * rho], v[4 * rho + 1]);
-          if (rs != r) D.d7a[o + d7_il(rs, m, ld)] = make_float2(sg * v[4 * rho + 2], sg * v[4 * rho + 3]);
-        }
+      for (int rho = 0; rho < 8; ++rho) {
+        if (8 * h + rho >= D.nreal) break;
+        const size_t o = (size_t)(8 * h + rho) * D.rstride + (size_t)j * D.prows * ld;
+        D.d7a[o + d7_il(r, m, ld)] = make_float2(v[4 * rho], v[4 * rho + 1]);
+        if (rs != r) D.d7a[o + d7_il(rs, m, ld)] = make_float2(sg * v[4 * rho + 2], sg * v[4 * rho + 3]);
       }
     }
   }
@@ -649,17 +768,16 @@ __device__ __forceinline__ void u0_unit(const TcDesc &D, int m, int rblk, unsign
   __syncthreads();
 }
 
-// CTA set-up and tear-down of the barriers (4 per half, `bars` holds 8) and the
+// CTA set-up and tear-down of the barriers (12 per part, `bars` holds 48) and the
 // tensor memory
-template <int NCOLS, int NH>
+template <int NCOLS, int NB, int NH>
 __device__ __forceinline__ void umma_open(UmmaCta &U, uint64_t *bars, uint32_t *tbase, int *abort) {
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int h = 0; h < NH; ++h) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[4 * h])));      // done[0]: the commit
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[4 * h + 1])));  // done[1]
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_u32(&bars[4 * h + 2])));  // full[0]: 4 warps
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_u32(&bars[4 * h + 3])));  // full[1]
+      for (int i = 0; i < 12; ++i)  // done: the commit; full: the group's warps; tile: the copy's arrival; free: one thread
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars[12 * h + i])),
+                     "r"((i == 2 || i == 3) ? 4 * NH / tc_groups(NH, NB) : 1));
     }
     asm volatile("fence.mbarrier_init.release.cluster;");
     *abort = 0;
@@ -674,22 +792,24 @@ __device__ __forceinline__ void umma_open(UmmaCta &U, uint64_t *bars, uint32_t *
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   U.tmem = *tbase;
   U.bars = smem_u32(&bars[0]);
-  U.count = 0;
-  U.count1 = 0;
+  U.c0 = U.c1 = U.c2 = U.c3 = 0;
+  U.g0 = U.g1 = 0;
   U.abort = abort;
   U.failed = false;
 }
 
 // NB: the buffers of the kernel's main unit type; the last block's commit of each
-// half covers every MMA issued before it.
+// group covers every MMA issued before it.
 template <int NCOLS, int NB, int NH>
 __device__ __forceinline__ void umma_close(const TcDesc &D, UmmaCta &U) {
   if (U.failed && threadIdx.x == 0) {
     atomicExch(D.err, 1);
     // own MMAs in flight (bounded)
-    if (U.count > 0) (void)mbar_wait(bar_done(U, buf_of<NB>(U.count - 1), 0), phase_of<NB>(U.count - 1), D.polls);
-    if (NH == 2 && U.count1 > 0)
-      (void)mbar_wait(bar_done(U, buf_of<NB>(U.count1 - 1), 1), phase_of<NB>(U.count1 - 1), D.polls);
+#pragma unroll
+    for (int gr = 0; gr < tc_groups(NH, NB); ++gr) {
+      const uint32_t c = group_count(U, gr);
+      if (c > 0) (void)mbar_wait(bar_done(U, buf_of<NB>(c - 1), gr), phase_of<NB>(c - 1), D.polls);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -700,7 +820,7 @@ __device__ __forceinline__ void umma_close(const TcDesc &D, UmmaCta &U) {
 template <int NDER, int MODE>
 struct Tc {
   static constexpr int NC = tc_cols(NDER);
-  static constexpr int NH = tc_halves(NDER + 1, MODE, NC);
+  static constexpr int NH = tc_parts(NDER + 1, MODE, NC);
   typedef TmemMap<NDER + 1, MODE, NC, NH> TM;
 };
 
@@ -708,13 +828,13 @@ template <int NDER, int MODE>
 __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MODE>::TM::ctas))
     legendre_spin2_umma(TcDesc D) {
   extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ __align__(8) uint64_t bars[8];
+  __shared__ __align__(8) uint64_t bars[48];
   __shared__ uint32_t tbase;
   __shared__ int abort_flag;
   typedef Tc<NDER, MODE> C;
   typedef typename C::TM TM;
   UmmaCta U;
-  umma_open<TM::cols, C::NH>(U, bars, &tbase, &abort_flag);
+  umma_open<TM::cols, TM::NB, C::NH>(U, bars, &tbase, &abort_flag);
   u2_unit<NDER, MODE, C::NC, TM::NB, C::NH>(D, blockIdx.y, blockIdx.x, sm, U);
   umma_close<TM::cols, TM::NB, C::NH>(D, U);
 }
@@ -723,20 +843,20 @@ __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MO
 // columns of the plan's order)
 template <int NDER, int MODE, int CNC>
 struct Tc0 {
-  static constexpr int NH = tc_halves(NDER + 1, MODE, CNC);
+  static constexpr int NH = tc_parts(NDER + 1, MODE, CNC);
   typedef TmemMap<NDER + 1, MODE, CNC, NH> TM;
 };
 template <int NDER, int MODE, int CNC>
 __global__ void __launch_bounds__(umma_threads(Tc0<NDER, MODE, CNC>::NH), (Tc0<NDER, MODE, CNC>::TM::ctas))
     legendre_spin0_umma(TcDesc D) {
   extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ __align__(8) uint64_t bars[8];
+  __shared__ __align__(8) uint64_t bars[48];
   __shared__ uint32_t tbase;
   __shared__ int abort_flag;
   typedef Tc0<NDER, MODE, CNC> C;
   typedef typename C::TM TM;
   UmmaCta U;
-  umma_open<TM::cols, C::NH>(U, bars, &tbase, &abort_flag);
+  umma_open<TM::cols, TM::NB, C::NH>(U, bars, &tbase, &abort_flag);
   u0_unit<NDER, MODE, CNC, TM::NB, C::NH>(D, blockIdx.y, blockIdx.x, sm, U);
   umma_close<TM::cols, TM::NB, C::NH>(D, U);
 }
@@ -745,13 +865,13 @@ __global__ void __launch_bounds__(umma_threads(Tc0<NDER, MODE, CNC>::NH), (Tc0<N
 // (descriptor, kind, m, ring block) are pre-sorted by cost; each CTA takes them in
 // order from an atomic counter until none is left (no waits between CTAs). Kinds:
 // 0 a spin-0 field at NDER, 1 the lensing potential (spin 0, NDER = 1), 2 spin 2.
-// Every kind's tensor-memory map fits the allocation of NDER's, with NDER's halves.
+// Every kind's tensor-memory map fits the allocation of NDER's, with NDER's parts.
 template <int NDER, int MODE>
 __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MODE>::TM::ctas))
     legendre_umma_persistent(const TcDesc *__restrict__ descs, const int4 *__restrict__ items, int nitems,
                              int *__restrict__ counter) {
   extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ __align__(8) uint64_t bars[8];
+  __shared__ __align__(8) uint64_t bars[48];
   __shared__ uint32_t tbase;
   __shared__ int abort_flag;
   __shared__ int cur;
@@ -761,7 +881,7 @@ __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MO
   typedef TmemMap<2, MODE, NC, NH> TM1;
   static_assert(TM1::A0 + NH * TM::NB * TM1::ASET <= TM::cols, "potential units fit the allocation");
   UmmaCta U;
-  umma_open<TM::cols, NH>(U, bars, &tbase, &abort_flag);
+  umma_open<TM::cols, TM::NB, NH>(U, bars, &tbase, &abort_flag);
   TcDesc D = descs[0];
   for (;;) {
     __syncthreads();  // the previous item's readers of `cur` are done
@@ -786,16 +906,16 @@ __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MO
 // Plan-time start table (see TcDesc): one CTA of 128 threads per unit runs the
 // recurrence block by block, without the contraction, until one of its rings has
 // reached scale 0 (a basis value that is not gated off), and records every ring's
-// state at the start of that block, bs. With state_mid it runs on to the first
-// block of the unit's second half, bmid = bs + (nblk - bs + 1) / 2, and records the
-// state there too. The launch kernels resume from these with the same arithmetic
-// (the same warps hold the same rings, so even the warp-uniform choices agree), so
+// state at the start of that block, bs. With state_mid it runs on and records the state at the
+// first block of the unit's quarters 1 .. 3 too. The launch kernels resume from these with the
+// same arithmetic (a warp holds the same 32 rings, so even the warp-uniform choices agree), so
 // their results are those of a run from l0. Units in which no ring contributes get
 // bstart = their block count.
 template <int NDER, bool SPIN2>
 __global__ void __launch_bounds__(kComputeThreads) tcstart_kernel(TcDesc D, int *__restrict__ bstart,
                                                                    float *__restrict__ state,
-                                                                   float *__restrict__ state_mid) {
+                                                                   float *__restrict__ state_mid,
+                                                                   long long mid_stride) {
   constexpr int NJ = NDER + 1;
   const int rblk = blockIdx.x, m = blockIdx.y, tid = threadIdx.x;
   const int l0 = unit_l0(m, SPIN2);
@@ -813,8 +933,23 @@ __global__ void __launch_bounds__(kComputeThreads) tcstart_kernel(TcDesc D, int 
   const bool mirror = SPIN2 && tid >= 64;
   const int qo = mirror ? 4 : 2;
   const size_t so = (size_t)unit * (2 * NJ + 1) * kComputeThreads + tid;
+  auto record = [&](float *st, const float (&sa)[NJ], const float (&sb)[NJ], int ssc) {
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      st[j * kComputeThreads] = sa[j];
+      st[(NJ + j) * kComputeThreads] = sb[j];
+    }
+    st[2 * NJ * kComputeThreads] = __int_as_float(ssc);
+  };
   int first = nblk, stop = nblk;
-  for (int blk = 0; blk < stop; ++blk) {
+  for (int blk = 0; blk <= stop; ++blk) {
+    if (first < nblk) {
+      // (a, b, sc) are the state at the start of this block
+#pragma unroll
+      for (int q = 1; q < 4; ++q)
+        if (blk == first + seg_first(nblk - first, q)) record(state_mid + (q - 1) * mid_stride + so, a, b, sc);
+    }
+    if (blk == stop) break;
     const float4 *stp = (const float4 *)(D.step + (b0 + blk) * step_stride(SPIN2));
     const float4 A0 = __ldg(stp), A1 = __ldg(stp + 1);
     const float4 C0 = __ldg(stp + qo), C1 = __ldg(stp + qo + 1);
@@ -832,32 +967,30 @@ __global__ void __launch_bounds__(kComputeThreads) tcstart_kernel(TcDesc D, int 
     // a ring can have contributed in this block only if its scale is 0 at the end
     if (first == nblk && __syncthreads_or(sc == 0)) {
       first = blk;
-      float *st = state + so;
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        st[j * kComputeThreads] = sa[j];
-        st[(NJ + j) * kComputeThreads] = sb[j];
-      }
-      st[2 * NJ * kComputeThreads] = __int_as_float(ssc);
+      record(state + so, sa, sb, ssc);
       if (!state_mid) break;
-      stop = first + (nblk - first + 1) / 2;  // bmid: record the state at its start
+      stop = first + seg_first(nblk - first, 3);
     }
-  }
-  if (state_mid && first < nblk) {
-    // (a, b, sc) are now the state at the start of block `stop` = bmid
-    float *st = state_mid + so;
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      st[j * kComputeThreads] = a[j];
-      st[(NJ + j) * kComputeThreads] = b[j];
-    }
-    st[2 * NJ * kComputeThreads] = __int_as_float(sc);
   }
   if (tid == 0) bstart[unit] = first;
 }
 
 // ---------------------------------------------------------------------------
 // plan-time and per-call tables
+
+// Leibniz coefficients e[j][i] = C(j, i) cos^(i)(theta) / L^i (leibniz_coefs), i = 1 .. j, of every ring,
+// [j (j - 1) / 2 + i - 1][ring]: the launch kernels' threads would form them in double once per
+// unit, on a pipe of two operations per cycle and SM
+__global__ void leib_table_kernel(RingTable rt, int nrings, int lmax, float *__restrict__ out) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= nrings) return;
+  Leib<float, TL_MAX_NDER> L;
+  leibniz_coefs<float, TL_MAX_NDER>(rt.z[r], rt.sint[r], 1.0 / (double)(lmax + 1), L);
+#pragma unroll
+  for (int j = 1; j <= TL_MAX_NDER; ++j)
+#pragma unroll
+    for (int i = 1; i <= j; ++i) out[(size_t)(j * (j - 1) / 2 + i - 1) * nrings + r] = L.e[j][i];
+}
 
 // step factors per block (layout of step_stride): A_{l+1} (8 floats), then for spin 0
 // A - 2 (8 floats), for spin 2 Qn = A - 2 + A C and Qs = A - 2 - A C (8 each), with
@@ -966,6 +1099,14 @@ __global__ void __launch_bounds__(256) tcprep_kernel(int lmax, int s, int nreal,
 // ---------------------------------------------------------------------------
 // launchers
 
+size_t tc_leib_bytes(const tl_plan *p) {
+  return sizeof(float) * (size_t)(TL_MAX_NDER * (TL_MAX_NDER + 1) / 2) * (size_t)p->nrings;
+}
+cudaError_t launch_tcleib(const tl_plan *p, float *out, cudaStream_t s) {
+  leib_table_kernel<<<(p->nrings + 127) / 128, 128, 0, s>>>(p->ring, p->nrings, p->lmax, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_tcstep(const tl_plan *p, int s, const long long *blkofs, const void *tab, float *out,
                           cudaStream_t st) {
   const int maxe = ((p->lmax + 8) / 8) * 8;
@@ -1002,12 +1143,13 @@ int tc_ring_blocks(const tl_plan *p, int spin) {
   return spin == 2 ? (2 * p->nside + 63) / 64 : (2 * p->nside + 127) / 128;
 }
 
-// Dynamic shared memory: two coefficient tiles and the spin-2 exchange area, raised
+// Dynamic shared memory: the coefficient tiles and the spin-2 exchange areas, raised
 // to the size that keeps the CTAs per SM within the tensor memory (512 columns per
-// SM): 4 CTAs (46 KB), 2 (76 KB) or 1 (114 KB).
+// SM): 3 CTAs (58 KB), 2 (76 KB) or 1 (114 KB).
 template <int CTAS, int NC, int NH> static size_t umma_smem() {
-  const size_t floor_b = CTAS >= 4 ? 46 * 1024 : CTAS == 2 ? 76 * 1024 : 114 * 1024;
-  const size_t need = xch_offset<NC, NH>() + kXchBytes;
+  static_assert(CTAS >= 1 && CTAS <= 3, "a floor for every CTA count");
+  const size_t floor_b = CTAS == 3 ? 58 * 1024 : CTAS == 2 ? 76 * 1024 : 114 * 1024;
+  const size_t need = xch_offset<NC, NH>() + NH * kXchBytes;
   return need > floor_b ? need : floor_b;
 }
 
@@ -1033,6 +1175,8 @@ static TcDesc make_desc(const tl_plan *p, int which, int nreal, const void *btil
   D.prows = d7_rows_il(p->nrings);
   D.err = p->dev_err;
   D.nrblk = tc_ring_blocks(p, spin);
+  D.leib = p->tc_leib;
+  D.mid_stride = (long long)(tc_start_state_bytes(p, which) / sizeof(float));
   D.bstart = which == 2 ? p->tc_bs2 : which == 1 ? p->tc_bsp : p->tc_bs0;
   D.state = which == 2 ? p->tc_st2 : which == 1 ? p->tc_stp : p->tc_st0;
   D.state_mid = which == 2 ? p->tc_sm2 : which == 1 ? p->tc_smp : p->tc_sm0;
@@ -1150,6 +1294,7 @@ cudaError_t launch_tcstart(const tl_plan *p, int which, int *bstart, float *stat
   D.bstart = nullptr;
   D.state = nullptr;
   D.state_mid = nullptr;
+  const long long ms = D.mid_stride;
   const int spin = which == 2 ? 2 : 0;
   const int nder = which == 1 ? 1 : p->tc_nder;
   dim3 grid(tc_ring_blocks(p, spin), p->mmax + 1);
@@ -1157,9 +1302,9 @@ cudaError_t launch_tcstart(const tl_plan *p, int which, int *bstart, float *stat
 #define CASE(n)                                                                                      \
   case n:                                                                                            \
     if (spin == 2)                                                                                   \
-      tcstart_kernel<n, true><<<grid, kComputeThreads, 0, s>>>(D, bstart, state, state_mid);         \
+      tcstart_kernel<n, true><<<grid, kComputeThreads, 0, s>>>(D, bstart, state, state_mid, ms);     \
     else                                                                                             \
-      tcstart_kernel<n, false><<<grid, kComputeThreads, 0, s>>>(D, bstart, state, state_mid);        \
+      tcstart_kernel<n, false><<<grid, kComputeThreads, 0, s>>>(D, bstart, state, state_mid, ms);    \
     return cudaGetLastError();
     TL_TC_ORDERS(CASE)
 #undef CASE
@@ -1172,13 +1317,6 @@ size_t tc_start_state_bytes(const tl_plan *p, int which) {
   const int nj = (which == 1 ? 1 : p->tc_nder) + 1;
   const size_t units = (size_t)(p->mmax + 1) * tc_ring_blocks(p, which == 2 ? 2 : 0);
   return units * (2 * nj + 1) * kComputeThreads * sizeof(float);
-}
-// Whether the kernels that run a start table's units split them into two halves
-// (and so need its midpoint table): which as in make_desc.
-bool tc_split(const tl_plan *p, int which) {
-  const int mode = tc_mode(p->precision), nc = tc_cols(p->tc_nder);
-  if (which == 1) return true;  // the potential's map (2 orders) always has room
-  return tc_halves(p->tc_nder + 1, mode, nc) == 2;
 }
 size_t tc_start_units(const tl_plan *p, int which) {
   return (size_t)(p->mmax + 1) * tc_ring_blocks(p, which == 2 ? 2 : 0);

@@ -100,7 +100,7 @@ static void free_plan(tl_plan *p) {
                   p->stage_out, p->gq, p->gq_count, p->phase,
                   p->tc_blk0, p->tc_blk2, p->tc_bm0, p->tc_bm2, p->tc_step0, p->tc_step2, p->tc_b0, p->tc_bp, p->tc_b2, p->dev_err,
                   p->tc_bs0, p->tc_bsp, p->tc_bs2, p->tc_st0, p->tc_stp, p->tc_st2, p->tc_sm0, p->tc_smp,
-                  p->tc_sm2,
+                  p->tc_sm2, p->tc_leib,
                   p->fft_rings, p->sy_rings, p->sy_corr, p->rest_rings};
   for (void *q : ptrs)
     if (q) cudaFree(q);
@@ -178,8 +178,8 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
       if (p->rest_ngroups < 0) return TL_ERR_UNSUPPORTED;
       TRY_CUDA(upload(&p->rest_rings, order, B));
     }
-    std::vector<float> corr(2 * (size_t)kSyCorr);
-    host_synth_window(&p->sy_win, corr.data(), corr.data() + kSyCorr);
+    const float *cw = host_synth_window(&p->sy_win);
+    std::vector<float> corr(cw, cw + 2 * (size_t)kSyCorr);
     TRY_CUDA(upload(&p->sy_rings, rings, B));
     TRY_CUDA(upload(&p->sy_corr, corr, B));
     for (int i = 0; i < p->sy_ngroups; ++i) sy_tw = sy_tw > (4 << p->sy_groups[i].lg) ? sy_tw : (4 << p->sy_groups[i].lg);
@@ -273,6 +273,8 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
       TRY_CUDA(launch_tcstep(p, 2, p->tc_blk2, p->tab2, p->tc_step2, 0));
       TRY_CUDA(dalloc(&p->tc_b2, bt * (size_t)(n2 > 0 ? n2 : 1), B));
     }
+    TRY_CUDA(dalloc((void **)&p->tc_leib, tc_leib_bytes(p), B));
+    TRY_CUDA(launch_tcleib(p, p->tc_leib, 0));
     // start tables: where each unit's first contribution begins (identical results)
     for (int which = 0; which < (pol ? 3 : 2); ++which) {
       int **bs = which == 0 ? &p->tc_bs0 : which == 1 ? &p->tc_bsp : &p->tc_bs2;
@@ -280,7 +282,7 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
       float **sm = which == 0 ? &p->tc_sm0 : which == 1 ? &p->tc_smp : &p->tc_sm2;
       TRY_CUDA(dalloc((void **)bs, sizeof(int) * tc_start_units(p, which), B));
       TRY_CUDA(dalloc((void **)st, tc_start_state_bytes(p, which), B));
-      if (tc_split(p, which)) TRY_CUDA(dalloc((void **)sm, tc_start_state_bytes(p, which), B));
+      TRY_CUDA(dalloc((void **)sm, 3 * tc_start_state_bytes(p, which), B));
       TRY_CUDA(launch_tcstart(p, which, *bs, *st, *sm, 0));
     }
     TRY_CUDA(cudaDeviceSynchronize());

@@ -407,17 +407,27 @@ static void kb_poly(int W, double beta, double c0, int D, float *out) {
 
 constexpr double kSigma10 = 1.65, kSigma8 = 2.0;
 
-// Window polynomials, and the correction tables: corr10[m] at m / 2^14 for m <= 2^13 /
-// kSigma10, corr8[m] for m <= 2^13 / kSigma8 (kSyCorr entries each)
-void host_synth_window(SyWindow *w, float *corr10, float *corr8) {
-  const double b10 = kb_beta(10, kSigma10), b8 = kb_beta(8, kSigma8);
-  for (int t = 0; t < 5; ++t) kb_poly(10, b10, t - 4.5, 8, w->c10[t]);
-  for (int t = 0; t < 4; ++t) kb_poly(8, b8, t - 3.5, 7, w->c8[t]);
-  for (int t = 0; t < 4; ++t) w->c8[t][8] = 0.0f;
-  for (int m = 0; m < kSyCorr; ++m) {
-    corr10[m] = (float)(1.0 / kb_transform(m / 16384.0, 10, b10));
-    corr8[m] = (float)(1.0 / kb_transform(m / 16384.0, 8, b8));
+// Window polynomials, and the correction tables: corr[m] of W = 10 at m / 2^14 for m <= 2^13 /
+// kSigma10, then of W = 8 for m <= 2^13 / kSigma8 (kSyCorr entries each). They depend on nothing:
+// formed once per process.
+struct SynthWindow {
+  SyWindow win;
+  float corr[2 * kSyCorr];
+  SynthWindow() {
+    const double b10 = kb_beta(10, kSigma10), b8 = kb_beta(8, kSigma8);
+    for (int t = 0; t < 5; ++t) kb_poly(10, b10, t - 4.5, 8, win.c10[t]);
+    for (int t = 0; t < 4; ++t) kb_poly(8, b8, t - 3.5, 7, win.c8[t]);
+    for (int t = 0; t < 4; ++t) win.c8[t][8] = 0.0f;
+    for (int m = 0; m < kSyCorr; ++m) {
+      corr[m] = (float)(1.0 / kb_transform(m / 16384.0, 10, b10));
+      corr[kSyCorr + m] = (float)(1.0 / kb_transform(m / 16384.0, 8, b8));
+    }
   }
+};
+const float *host_synth_window(SyWindow *w) {
+  static const SynthWindow s;  // initialised by the first thread to get here
+  *w = s.win;
+  return s.corr;
 }
 
 // Group of one ring, by its length and band (mcut: its coefficients beyond are zero):
