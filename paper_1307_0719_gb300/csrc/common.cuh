@@ -92,11 +92,12 @@ struct tl_plan {
   // single-precision ring synthesis: its groups, and those of the rings it does not take
   int sy_ngroups, rest_ngroups;
   tl::SyGroup sy_groups[TL_MAX_SY_GROUPS];
-  int4 *sy_rings;       // {ring, band, fold, 0} by group (device)
+  int4 *sy_rings;       // {ring, band, fold, mcut} by group (device)
   float *sy_corr;       // [2][kSyCorr] corrections of the two windows (device)
   tl::SyWindow sy_win;
   int *rest_rings;      // ring indices of rest_groups (device)
   tl::FftGroup rest_groups[TL_MAX_FFT_GROUPS];
+  int *mcut;            // [nrings] largest m that is not held at zero on the ring (device; NULL: not known)
   // workspace
   void *tab0, *tab2;    // plan-time step tables {k_l, A_{l+1}} for spin 0 and spin 2
   void *rec_T, *rec_P, *rec_QU; // coefficient records
@@ -160,6 +161,9 @@ cudaError_t launch_prep_spin0(const tl_plan *p, const double *alm, const double 
 cudaError_t launch_prep_spin2(const tl_plan *p, const double *alm_E, const double *alm_B, cudaStream_t s);
 cudaError_t launch_legendre_spin0(const tl_plan *p, int nder, bool phi, void *d7, void *d7p, cudaStream_t s);
 cudaError_t launch_legendre_spin2(const tl_plan *p, int nder, cudaStream_t s);
+// their single-precision forms (legendre_f32.cu)
+cudaError_t launch_legendre_spin0_f32(const tl_plan *p, int nder, bool phi, void *d7, void *d7p, cudaStream_t s);
+cudaError_t launch_legendre_spin2_f32(const tl_plan *p, int nder, cudaStream_t s);
 
 // Pixel-tiled layout of the plan's derivative maps (d3): [tile][map][kD3Tile], one
 // tile holding every map's values of kD3Tile consecutive pixels, so that the gather's
@@ -262,8 +266,9 @@ size_t ringfft_smem_bytes(const tl_plan *p);
 // (of the rings with use[r] != 0 only, when use is given)
 int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGroup *groups, int *order,
                     const unsigned char *use = nullptr);
-// mcut[r]: the largest m whose coefficients can be non-zero on ring r at band limit lmax
-void host_ring_bands(int nside, int lmax, const double *sint, const double *z, int *mcut);
+// mcut[r]: the largest m whose coefficients can be non-zero on ring r at band limit lmax, functions
+// below 2^-h being held at zero
+void host_ring_bands(int nside, int lmax, int h, const double *sint, const double *z, int *mcut);
 struct JobList;
 const float *host_synth_window(SyWindow *w);  // returns [2][kSyCorr] corrections
 int host_synth_groups(int nside, int nrings, const int *nphi, const int *mcut, SyGroup *groups, int4 *rings, int *rest,

@@ -1,5 +1,5 @@
-// Legendre stage kernels, their plan-time step tables and the per-call
-// coefficient preparation. See legendre.cuh for the mathematics (Naess & Louis
+// Legendre stage kernels (in double precision; single precision in legendre_f32.cu), their
+// plan-time step tables and the per-call coefficient preparation. See legendre.cuh for the mathematics (Naess & Louis
 // 2013, Sec. II.B: the derivative maps of Eq. 4).
 //
 // Normalised recurrence. With lam_l = k_l mu_l and k_{l+1} = beta_{l+1} k_{l-1}
@@ -143,6 +143,7 @@ __global__ void prep_spin2_kernel(int lmax, const double *__restrict__ almE, con
 template <typename T, int NDER, bool PHI>
 __global__ void __launch_bounds__(128) legendre_spin0_kernel(RingTable rt, const double *__restrict__ lnorm0,
                                                              int nside, int lmax, int mmax, int nrings,
+                                                             const int *__restrict__ mcut,
                                                              const Rec0<T> *__restrict__ rec,
                                                              const typename RealTraits<T>::T2 *__restrict__ recp,
                                                              typename RealTraits<T>::T2 *__restrict__ d7,
@@ -152,6 +153,8 @@ __global__ void __launch_bounds__(128) legendre_spin0_kernel(RingTable rt, const
   const int m = blockIdx.y;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;  // north ring index 0 .. 2N-1
   if (r >= 2 * nside) return;
+  // rings that never leave zero at this m (host_ring_bands): no steps
+  const int top = (!mcut || __any_sync(__activemask(), m <= mcut[r])) ? lmax : -1;
   const double invL = 1.0 / (double)(lmax + 1);
   const double x = rt.z[r], st = rt.sint[r];
   Leib<T, NDER> LC;
@@ -176,7 +179,7 @@ __global__ void __launch_bounds__(128) legendre_spin0_kernel(RingTable rt, const
   Rec0<T> cn = rm[m];
   T2 pn;
   if (PHI) pn = pm[m];
-  for (int l = m;; l += 2) {
+  for (int l = m; l <= top; l += 2) {
     // ---- even l - m
     {
       const Rec0<T> c = cn;
@@ -296,6 +299,7 @@ __device__ __forceinline__ void spin2_sweep(const Rec2<T> *__restrict__ rm, int 
 template <typename T, int NDER, int RP>
 __global__ void __launch_bounds__(2 * RP) legendre_spin2_kernel(RingTable rt, const double *__restrict__ lnorm0,
                                                                 int nside, int lmax, int mmax, int nrings,
+                                                                const int *__restrict__ mcut,
                                                                 const Rec2<T> *__restrict__ rec,
                                                                 typename RealTraits<T>::T2 *__restrict__ d7q,
                                                                 typename RealTraits<T>::T2 *__restrict__ d7u) {
@@ -313,7 +317,9 @@ __global__ void __launch_bounds__(2 * RP) legendre_spin2_kernel(RingTable rt, co
 #pragma unroll
   for (int j = 0; j <= NDER; ++j) s1r[j] = s1i[j] = s2r[j] = s2i[j] = (T)0;
 
-  if (active) {
+  // rings that never leave zero at this m (host_ring_bands): no steps
+  const bool live = __any_sync(0xffffffffu, active && (!mcut || m <= mcut[r]));
+  if (active && live) {
     const double x = rt.z[r], st = rt.sint[r];
     Leib<T, NDER> LC;
     leibniz_coefs<T, NDER>(x, st, invL, LC);
@@ -402,7 +408,7 @@ static cudaError_t leg0(const tl_plan *p, void *d7, void *d7p, cudaStream_t s) {
   const int threads = 64;
   dim3 grid((2 * p->nside + threads - 1) / threads, p->mmax + 1);
   legendre_spin0_kernel<T, NDER, PHI><<<grid, threads, 0, s>>>(
-      p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings, (const Rec0<T> *)p->rec_T,
+      p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings, p->mcut, (const Rec0<T> *)p->rec_T,
       (const T2 *)p->rec_P, (T2 *)d7, (T2 *)d7p);
   return cudaGetLastError();
 }
@@ -412,7 +418,7 @@ static cudaError_t leg2(const tl_plan *p, cudaStream_t s) {
   constexpr int RP = 32;
   dim3 grid((2 * p->nside + RP - 1) / RP, p->mmax + 1);
   legendre_spin2_kernel<T, NDER, RP><<<grid, 2 * RP, 0, s>>>(
-      p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings, (const Rec2<T> *)p->rec_QU,
+      p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings, p->mcut, (const Rec2<T> *)p->rec_QU,
       (typename RealTraits<T>::T2 *)p->d7_Q, (typename RealTraits<T>::T2 *)p->d7_U);
   return cudaGetLastError();
 }
@@ -448,13 +454,12 @@ static cudaError_t leg2_dispatch(const tl_plan *p, int nder, cudaStream_t s) {
 // Spin-0 stage on the prepared T records (into d7) and, when phi is set, the
 // potential's j <= 1 planes (into d7p) from the same recurrence.
 cudaError_t launch_legendre_spin0(const tl_plan *p, int nder, bool phi, void *d7, void *d7p, cudaStream_t s) {
-  if (p->precision == TL_FP64)
-    return phi ? leg0_dispatch<double, true>(p, nder, d7, d7p, s) : leg0_dispatch<double, false>(p, nder, d7, d7p, s);
-  return phi ? leg0_dispatch<float, true>(p, nder, d7, d7p, s) : leg0_dispatch<float, false>(p, nder, d7, d7p, s);
+  if (p->precision != TL_FP64) return launch_legendre_spin0_f32(p, nder, phi, d7, d7p, s);
+  return phi ? leg0_dispatch<double, true>(p, nder, d7, d7p, s) : leg0_dispatch<double, false>(p, nder, d7, d7p, s);
 }
 
 cudaError_t launch_legendre_spin2(const tl_plan *p, int nder, cudaStream_t s) {
-  return p->precision == TL_FP64 ? leg2_dispatch<double>(p, nder, s) : leg2_dispatch<float>(p, nder, s);
+  return p->precision == TL_FP64 ? leg2_dispatch<double>(p, nder, s) : launch_legendre_spin2_f32(p, nder, s);
 }
 
 }  // namespace tl

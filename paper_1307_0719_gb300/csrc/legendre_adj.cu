@@ -62,7 +62,8 @@ __device__ __forceinline__ void flush_window(T (*win)[WV + 1], int nl, long long
 
 template <typename T, int NDER, bool PHI>
 __global__ void __launch_bounds__(128) legendre_adj0_kernel(RingTable rt, const double *__restrict__ lnorm0,
-                                                            int nside, int lmax, int mmax, int nrings, int nder_T,
+                                                            int nside, int lmax, int mmax, int nrings,
+                                                            const int *__restrict__ mcut, int nder_T,
                                                             const typename RealTraits<T>::T2 *__restrict__ tab,
                                                             const typename RealTraits<T>::T2 *__restrict__ FT,
                                                             const typename RealTraits<T>::T2 *__restrict__ FP,
@@ -75,6 +76,10 @@ __global__ void __launch_bounds__(128) legendre_adj0_kernel(RingTable rt, const 
   const int rn = blockIdx.x * NT + tid;
   const bool active = rn < 2 * nside && m <= mmax;
   const int r = active ? rn : 0;
+  // a block none of whose rings leaves zero at this m (host_ring_bands) adds nothing; a warp of
+  // such rings runs no steps
+  const bool live = __any_sync(0xffffffffu, active && (!mcut || m <= mcut[r]));
+  if (!__syncthreads_or(live)) return;
   const int rs = nrings - 1 - r;
   const double invL = 1.0 / (double)(lmax + 1);
   const size_t ld = (size_t)(mmax + 1);
@@ -152,9 +157,11 @@ __global__ void __launch_bounds__(128) legendre_adj0_kernel(RingTable rt, const 
         lb += W;
       }
       if (l == lmax) break;
-      const T Q = tm[l].y;
-      rec_step<T, NDER, 1>(a, b, LC, X, w, (T)2 + Q, Q);
-      rescale<T, NDER>(a, b, b[0], sc);
+      if (live) {
+        const T Q = tm[l].y;
+        rec_step<T, NDER, 1>(a, b, LC, X, w, (T)2 + Q, Q);
+        rescale<T, NDER>(a, b, b[0], sc);
+      }
     }
     // ---- odd l - m
     {
@@ -185,9 +192,11 @@ __global__ void __launch_bounds__(128) legendre_adj0_kernel(RingTable rt, const 
         lb += W;
       }
       if (l + 1 == lmax) break;
-      const T Q = tm[l + 1].y;
-      rec_step<T, NDER, 1>(a, b, LC, X, w, (T)2 + Q, Q);
-      rescale<T, NDER>(a, b, b[0], sc);
+      if (live) {
+        const T Q = tm[l + 1].y;
+        rec_step<T, NDER, 1>(a, b, LC, X, w, (T)2 + Q, Q);
+        rescale<T, NDER>(a, b, b[0], sc);
+      }
     }
   }
 }
@@ -202,7 +211,7 @@ __device__ __forceinline__ void adj2_sweep(const Rec2<T> *__restrict__ rm, int l
                                            const Leib<T, NDER> &LC, T X, T w, T (&a)[NDER + 1], T (&b)[NDER + 1],
                                            int &sc, const T (&u1r)[NDER + 1], const T (&u1i)[NDER + 1],
                                            const T (&u2r)[NDER + 1], const T (&u2i)[NDER + 1],
-                                           T (*win)[WV + 1], double *accE, double *accB) {
+                                           T (*win)[WV + 1], double *accE, double *accB, bool live) {
   constexpr int NT = 128, V = 4, W = WV / V;
   const int t = threadIdx.x;
   int lb = l0;
@@ -234,9 +243,11 @@ __device__ __forceinline__ void adj2_sweep(const Rec2<T> *__restrict__ rm, int l
         lb += W;
       }
       if (ll == lmax) return;
-      const Rec2<T> c = rm[ll];
-      rec_step<T, NDER, SG>(a, b, LC, X + c.cterm, w, c.A, SG > 0 ? c.Qn : c.Qs);
-      rescale<T, NDER>(a, b, b[0], sc);
+      if (live) {
+        const Rec2<T> c = rm[ll];
+        rec_step<T, NDER, SG>(a, b, LC, X + c.cterm, w, c.A, SG > 0 ? c.Qn : c.Qs);
+        rescale<T, NDER>(a, b, b[0], sc);
+      }
     }
     if (l + 1 >= lmax) return;
   }
@@ -245,6 +256,7 @@ __device__ __forceinline__ void adj2_sweep(const Rec2<T> *__restrict__ rm, int l
 template <typename T, int NDER>
 __global__ void __launch_bounds__(128) legendre_adj2_kernel(RingTable rt, const double *__restrict__ lnorm0,
                                                             int nside, int lmax, int mmax, int nrings,
+                                                            const int *__restrict__ mcut,
                                                             const Rec2<T> *__restrict__ rec,
                                                             const typename RealTraits<T>::T2 *__restrict__ FQ,
                                                             const typename RealTraits<T>::T2 *__restrict__ FU,
@@ -261,6 +273,9 @@ __global__ void __launch_bounds__(128) legendre_adj2_kernel(RingTable rt, const 
   const bool active = rn < 2 * nside && m <= mmax && !(mirror && equator);
   const int r = rn < 2 * nside ? (mirror ? nrings - 1 - rn : rn) : 0;
   const int rp = nrings - 1 - r;  // partner (mirror) ring
+  // (as for spin 0)
+  const bool live = __any_sync(0xffffffffu, active && (!mcut || m <= mcut[r]));
+  if (!__syncthreads_or(live)) return;
   const double invL = 1.0 / (double)(lmax + 1);
   const size_t ld = (size_t)(mmax + 1);
   const int mm = m <= mmax ? m : mmax;
@@ -302,9 +317,11 @@ __global__ void __launch_bounds__(128) legendre_adj2_kernel(RingTable rt, const 
   // mirror threads (cos th < 0) are warps 2 and 3; the window flushes inside keep
   // every thread of the block in step, so both branches run the same l sequence
   if (mirror)
-    adj2_sweep<T, NDER, -1, WV>(rm, l0, m, lmax, base, LC, X, w, a, b, sc, u1r, u1i, u2r, u2i, win, accE, accB);
+    adj2_sweep<T, NDER, -1, WV>(rm, l0, m, lmax, base, LC, X, w, a, b, sc, u1r, u1i, u2r, u2i, win, accE, accB,
+                                live);
   else
-    adj2_sweep<T, NDER, 1, WV>(rm, l0, m, lmax, base, LC, X, w, a, b, sc, u1r, u1i, u2r, u2i, win, accE, accB);
+    adj2_sweep<T, NDER, 1, WV>(rm, l0, m, lmax, base, LC, X, w, a, b, sc, u1r, u1i, u2r, u2i, win, accE, accB,
+                                live);
 }
 
 // Final scaling: abar = k_l acc; B's accumulator holds f with Bbar = -i k f;
@@ -349,7 +366,7 @@ static cudaError_t adj0(const tl_plan *p, int nder_T, const void *FT, const void
   typedef typename RealTraits<T>::T2 T2;
   dim3 grid((2 * p->nside + 127) / 128, p->mmax + 1);
   legendre_adj0_kernel<T, NDER, PHI><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax,
-                                                          p->nrings, nder_T, (const T2 *)p->tab0, (const T2 *)FT,
+                                                          p->nrings, p->mcut, nder_T, (const T2 *)p->tab0, (const T2 *)FT,
                                                           (const T2 *)FP, aT, aP);
   return cudaGetLastError();
 }
@@ -384,7 +401,7 @@ template <typename T, int NDER>
 static cudaError_t adj2(const tl_plan *p, const void *FQ, const void *FU, double *aE, double *aB, cudaStream_t s) {
   typedef typename RealTraits<T>::T2 T2;
   dim3 grid((2 * p->nside + 63) / 64, p->mmax + 1);
-  legendre_adj2_kernel<T, NDER><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings,
+  legendre_adj2_kernel<T, NDER><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings, p->mcut,
                                                      (const Rec2<T> *)p->rec_QU, (const T2 *)FQ, (const T2 *)FU, aE,
                                                      aB);
   return cudaGetLastError();

@@ -270,6 +270,9 @@ struct TcDesc {
   const float *state_mid;
   long long mid_stride;
   const float *leib;             // Leibniz coefficients e[j][i] per ring (leib_table_kernel)
+  // [nrings] or NULL: coefficients of m > mcut[ring] (zeros) are not stored, because the ring
+  // synthesis does not read them
+  const int *mcut;
   int nrblk;
   int polls;  // polls of every mbarrier wait before it gives up (bounded waits)
   int stall;  // self-test: the compute warps withhold their arrivals, so waits run out
@@ -686,13 +689,15 @@ __device__ __forceinline__ void u2_unit(const TcDesc &D, int m, int rblk, unsign
   const int tid = threadIdx.x, warp = tid >> 5;
   const int nblk = run_blocks<NDER, MODE, NC, NB, true, NH>(D, m, rblk, sm, U);
   if (U.failed) return;
-  if (warp < 4 * NH) {
-    const int part = warp >> 2, t = tid & (kComputeThreads - 1);
-    const int rn = rblk * 64 + (t & 63);
-    const bool active = rn < 2 * D.nside;
-    const bool mirror = t >= 64;
-    const int r = active ? (mirror ? D.nrings - 1 - rn : rn) : 0;
-    const bool writer = active && m <= D.mmax && !(mirror && rn == D.nrings - 1 - rn);  // equator: north thread
+  const int part = warp >> 2, t = tid & (kComputeThreads - 1);
+  const int rn = rblk * 64 + (t & 63);
+  const bool active = rn < 2 * D.nside;
+  const bool mirror = t >= 64;
+  const int r = active ? (mirror ? D.nrings - 1 - rn : rn) : 0;
+  const bool writer = warp < 4 * NH && active && m <= D.mmax &&
+                      !(mirror && rn == D.nrings - 1 - rn) &&  // equator: the north thread writes it
+                      (!D.mcut || m <= D.mcut[r]);
+  if (__syncthreads_or(writer) && warp < 4 * NH) {
     const int partner = t ^ 64;
     const size_t ld = (size_t)(D.mmax + 1);
     // [128][kXchRow]: S2 (4 rho + 2, 3) of every ring
@@ -736,10 +741,10 @@ __device__ __forceinline__ void u0_unit(const TcDesc &D, int m, int rblk, unsign
   const int tid = threadIdx.x, warp = tid >> 5;
   const int nblk = run_blocks<NDER, MODE, NC, NB, false, NH>(D, m, rblk, sm, U);
   if (U.failed) return;
-  if (warp < 4 * NH) {
-    const int part = warp >> 2, t = tid & (kComputeThreads - 1);
-    const int rn = rblk * 128 + t;
-    const bool active = rn < 2 * D.nside && m <= D.mmax;
+  const int part = warp >> 2, t = tid & (kComputeThreads - 1);
+  const int rn = rblk * 128 + t;
+  const bool active = warp < 4 * NH && rn < 2 * D.nside && m <= D.mmax && (!D.mcut || m <= D.mcut[rn]);
+  if (__syncthreads_or(active) && warp < 4 * NH) {
     const int r = active ? rn : 0;
     const int rs = D.nrings - 1 - r;
     const size_t ld = (size_t)(D.mmax + 1);
@@ -1175,6 +1180,7 @@ static TcDesc make_desc(const tl_plan *p, int which, int nreal, const void *btil
   D.prows = d7_rows_il(p->nrings);
   D.err = p->dev_err;
   D.nrblk = tc_ring_blocks(p, spin);
+  D.mcut = p->sy_ngroups > 0 && p->rest_ngroups == 0 ? p->mcut : nullptr;
   D.leib = p->tc_leib;
   D.mid_stride = (long long)(tc_start_state_bytes(p, which) / sizeof(float));
   D.bstart = which == 2 ? p->tc_bs2 : which == 1 ? p->tc_bsp : p->tc_bs0;

@@ -101,7 +101,7 @@ static void free_plan(tl_plan *p) {
                   p->tc_blk0, p->tc_blk2, p->tc_bm0, p->tc_bm2, p->tc_step0, p->tc_step2, p->tc_b0, p->tc_bp, p->tc_b2, p->dev_err,
                   p->tc_bs0, p->tc_bsp, p->tc_bs2, p->tc_st0, p->tc_stp, p->tc_st2, p->tc_sm0, p->tc_smp,
                   p->tc_sm2, p->tc_leib,
-                  p->fft_rings, p->sy_rings, p->sy_corr, p->rest_rings};
+                  p->fft_rings, p->mcut, p->sy_rings, p->sy_corr, p->rest_rings};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   if (p->timing)
@@ -163,10 +163,12 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
   const char *rr = getenv("TAYLENS_RING_FFT");  // "shared": the general kernel for every ring
   p->ring_reg = (rr && strcmp(rr, "shared") == 0) ? 0 : 1;
   int sy_tw = 0;
+  std::vector<int> mcut(p->nrings);
+  host_ring_bands(nside, lmax, precision == TL_FP64 ? 200 : 32, h.sint.data(), h.z.data(), mcut.data());
+  TRY_CUDA(upload(&p->mcut, mcut, B));
   if (precision != TL_FP64 && p->ring_reg) {
-    std::vector<int> mcut(p->nrings), rest(p->nrings), order(p->nrings);
+    std::vector<int> rest(p->nrings), order(p->nrings);
     std::vector<int4> rings(p->nrings);
-    host_ring_bands(nside, lmax, h.sint.data(), h.z.data(), mcut.data());
     int nrest = 0;
     p->sy_ngroups = host_synth_groups(nside, p->nrings, h.nphi.data(), mcut.data(), p->sy_groups, rings.data(),
                                       rest.data(), &nrest);

@@ -18,8 +18,8 @@
 // the ring's own length per map; Bluestein's chirp-z convolution, exact for any length, takes
 // four of 2 to 4 times the sub-sequence length each (per map of a packed pair).
 //
-// The rows of F are zero beyond the ring's band (see host_ring_bands): a function whose
-// coefficients all lie below 2^-32 is gated off by the Legendre stage. Rows are staged
+// The rows of F are zero beyond the ring's mcut (see host_ring_bands): the Legendre stage holds
+// functions below 2^-32 at zero. Nothing beyond is read. Rows are staged
 // once per plane in shared memory, scaled by the window's correction, and multiplied by
 // i m / L from one phi-derivative to the next. Where the band limit exceeds half the
 // ring's length the aliases are folded while staging (per map, since (m / L)^k is not a
@@ -82,7 +82,7 @@ struct SyArgs {
   const long long *first;
   const double *phi0;
   const float *rsinf;
-  const int4 *rings;    // {ring, band, fold, 0}
+  const int4 *rings;    // {ring, band, fold, mcut}
   const float2 *tw;     // e^{-2 pi i k / TW}, k < TW / 2
   const float *corr;    // 1 / (window's transform) at m / (finest grid)
   int lgtw, mmax, rounds, chunks, rowcap;
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(SyCfg<LG, MODE>::NT, SyCfg<LG, MODE>::CTAS)
         const float2 *FR = job_row<float2>(J, r, A.mmax, fs);
         if (fold) {
           for (int m = sm0; m <= band; m += sms) {
-            float2 v = sy_fold(FR, fs, m, N, A.mmax, k, A.invL, shifted);
+            float2 v = sy_fold(FR, fs, m, N, R.w, k, A.invL, shifted);
             if (INTERP) {
               const float c = __ldg(A.corr + m * cstep);
               v = f2(v.x * c, v.y * c);
@@ -464,7 +464,7 @@ static int synth_key(int nside, int nphi, int mcut, int *band, int *fold) {
   return key;
 }
 
-// Ring groups of the synthesis kernels: rings[] = {ring, band, fold, 0} by group, longest
+// Ring groups of the synthesis kernels: rings[] = {ring, band, fold, mcut} by group, longest
 // rings first within a group. Rings that no grid fits go to rest[] (*nrest). Returns the number of groups.
 int host_synth_groups(int nside, int nrings, const int *nphi, const int *mcut, SyGroup *groups, int4 *rings, int *rest,
                       int *nrest) {
@@ -478,7 +478,7 @@ int host_synth_groups(int nside, int nrings, const int *nphi, const int *mcut, S
       const int r = (nrings / 2) + ((d & 1) ? (d + 1) / 2 : -(d / 2));
       int band, fold;
       if (synth_key(nside, nphi[r], mcut[r], &band, &fold) != key) continue;
-      rings[n++] = make_int4(r, band, fold, 0);
+      rings[n++] = make_int4(r, band, fold, mcut[r]);
       if (band > cap) cap = band;
     }
     if (n == first) continue;

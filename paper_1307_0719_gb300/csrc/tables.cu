@@ -172,15 +172,16 @@ int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGr
   return n == want ? ng : -1;
 }
 
-// The Legendre stage holds a function of (l, m) at zero until it reaches 2^-32. Beyond the
-// turning point sin theta_t = m / L (L = lmax + 1/2) the largest l is damped by e^-S,
+// The Legendre stage holds a function of (l, m) at zero until it reaches 2^-h (h = 32 in
+// single precision, 200 in double). Beyond the turning point sin theta_t = m / L (L = lmax + 1/2)
+// the largest l is damped by e^-S,
 //   S = int_theta^theta_t sqrt(m^2 / sin^2 t - L^2) dt
 //     = m artanh(R / (m cos theta)) - L artanh(R / (L cos theta)),  R^2 = m^2 - L^2 sin^2 theta
 // (the first-order WKB exponent; smaller l are damped more). Its prefactor is of order one:
-// S = 26 against 32 ln 2 = 22.2, and three more in m for the spin's shift, leave no ring of
-// any (Nside, lmax) tried with a non-zero coefficient beyond (spin 0 and 2; slack about 7).
-void host_ring_bands(int nside, int lmax, const double *sint, const double *z, int *mcut) {
-  const double L = lmax + 0.5;
+// S = h ln 2 + 3.8, and three more in m for the spin's shift, leave no ring of any (Nside, lmax)
+// tried with a non-zero coefficient beyond (spin 0 and 2; slack about 7).
+void host_ring_bands(int nside, int lmax, int h, const double *sint, const double *z, int *mcut) {
+  const double L = lmax + 0.5, most = h * 0.69314718055994531 + 3.8;
   const int nr = 4 * nside - 1;
   for (int r = 0; r < 2 * nside; ++r) {
     const double s = sint[r], c = fabs(z[r]);
@@ -192,12 +193,12 @@ void host_ring_bands(int nside, int lmax, const double *sint, const double *z, i
       return m * atanh(a) - L * atanh(b);
     };
     int lo = 0, hi = lmax;
-    if (damp(lmax) < 26.0) {
+    if (damp(lmax) < most) {
       lo = lmax;
     } else {
       while (hi - lo > 1) {
         const int k = (lo + hi) / 2;
-        if (damp(k) < 26.0) lo = k;
+        if (damp(k) < most) lo = k;
         else hi = k;
       }
       lo = lo + 3 < lmax ? lo + 3 : lmax;

@@ -38,7 +38,15 @@ def test_derivs_spin0_vs_oracle(nside, lmax, order):
         assert rel_rms(out[i], ref[i]) < TOL, (i, rel_rms(out[i], ref[i]))
 
 
-@pytest.mark.parametrize("nside,lmax,order", [(2, 16, 3), (32, 75, 4), (64, 200, 2), (128, 300, 1)])
+def test_spin2_below_its_lowest_l_is_zero():
+    """lmax 1 holds no spin-2 harmonics."""
+    s = sky(2, 1, pol=True, seeds=(11, 12, 1))
+    d = to_dev(s)
+    out = api.synth_derivs(2, 1, 2, torch.cat([d["E"], d["B"]]), 2, api.MIXED_FP32)
+    assert torch.count_nonzero(out) == 0
+
+
+@pytest.mark.parametrize("nside,lmax,order", [(2, 2, 2), (2, 16, 3), (32, 75, 4), (64, 200, 2), (128, 300, 1)])
 def test_derivs_spin2_vs_oracle(nside, lmax, order):
     s = sky(nside, lmax, pol=True, seeds=(11, 12, 1), b_scale=0.6)
     ref = OL.derivative_maps(nside, lmax, order, alm_E=s["E"], alm_B=s["B"])
