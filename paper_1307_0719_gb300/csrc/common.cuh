@@ -93,6 +93,7 @@ struct tl_plan {
   int sy_ngroups, rest_ngroups;
   tl::SyGroup sy_groups[TL_MAX_SY_GROUPS];
   int4 *sy_rings;       // {ring, band, fold, mcut} by group (device)
+  float4 *sy_tw4;       // twiddles of the synthesis transforms (host_synth_twiddles)
   float *sy_corr;       // [2][kSyCorr] corrections of the two windows (device)
   tl::SyWindow sy_win;
   int *rest_rings;      // ring indices of rest_groups (device)
@@ -270,6 +271,8 @@ int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGr
 // below 2^-h being held at zero
 void host_ring_bands(int nside, int lmax, int h, const double *sint, const double *z, int *mcut);
 struct JobList;
+// entries (eight floats each) of the synthesis kernels' twiddle table, filled when out is given
+int host_synth_twiddles(float *out);
 const float *host_synth_window(SyWindow *w);  // returns [2][kSyCorr] corrections
 int host_synth_groups(int nside, int nrings, const int *nphi, const int *mcut, SyGroup *groups, int4 *rings, int *rest,
                       int *nrest);

@@ -101,7 +101,7 @@ static void free_plan(tl_plan *p) {
                   p->tc_blk0, p->tc_blk2, p->tc_bm0, p->tc_bm2, p->tc_step0, p->tc_step2, p->tc_b0, p->tc_bp, p->tc_b2, p->dev_err,
                   p->tc_bs0, p->tc_bsp, p->tc_bs2, p->tc_st0, p->tc_stp, p->tc_st2, p->tc_sm0, p->tc_smp,
                   p->tc_sm2, p->tc_leib,
-                  p->fft_rings, p->mcut, p->sy_rings, p->sy_corr, p->rest_rings};
+                  p->fft_rings, p->mcut, p->sy_rings, p->sy_corr, p->sy_tw4, p->rest_rings};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   if (p->timing)
@@ -184,6 +184,9 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
     std::vector<float> corr(cw, cw + 2 * (size_t)kSyCorr);
     TRY_CUDA(upload(&p->sy_rings, rings, B));
     TRY_CUDA(upload(&p->sy_corr, corr, B));
+    std::vector<float> tw4(8 * (size_t)host_synth_twiddles(nullptr));
+    host_synth_twiddles(tw4.data());
+    TRY_CUDA(upload((float **)&p->sy_tw4, tw4, B));
     for (int i = 0; i < p->sy_ngroups; ++i) sy_tw = sy_tw > (4 << p->sy_groups[i].lg) ? sy_tw : (4 << p->sy_groups[i].lg);
   }
 

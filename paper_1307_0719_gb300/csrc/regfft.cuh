@@ -122,6 +122,41 @@ __device__ __forceinline__ void dft_small(float2 *a) {
 __device__ __forceinline__ int rpad(int a) { return a + (a >> 4); }
 __device__ __forceinline__ float2 conj_if(float2 a, bool c) { return c ? f2(a.x, -a.y) : a; }
 
+// Where a pass takes W_L^j, W_L^2j, W_L^4j and W_L^8j (j < L / 16, sign DIR) from:
+// the plan's table tw[k] = e^{-2 pi i k / TW}, k < TW / 2
+template <int DIR> struct TwidTable {
+  const float2 *__restrict__ tw;
+  int lgtw;
+  template <int LG, int P>
+  __device__ __forceinline__ void get(int j, float2 &w1, float2 &w2, float2 &w4, float2 &w8) const {
+    const int s = j << (lgtw - (LG - 4 * P));
+    const bool cj = DIR > 0;
+    w1 = conj_if(__ldg(tw + s), cj);
+    w2 = conj_if(__ldg(tw + 2 * s), cj);
+    w4 = conj_if(__ldg(tw + 4 * s), cj);
+    w8 = conj_if(__ldg(tw + 8 * s), cj);
+  }
+};
+// or a table of the four side by side per pass (DIR = +1), pass by pass: 32 bytes per j, so that a
+// warp's loads touch 8 lines a pass (their scattered entries of tw lie in up to 88)
+struct TwidPacked {
+  const float4 *__restrict__ t;
+  // entries of the passes before pass P
+  template <int LG> __host__ __device__ static constexpr int offset(int P) {
+    int n = 0;
+    for (int i = 0; i < P; ++i) n += 1 << (LG - 4 * i - 4);
+    return n;
+  }
+  template <int LG, int P>
+  __device__ __forceinline__ void get(int j, float2 &w1, float2 &w2, float2 &w4, float2 &w8) const {
+    const float4 a = __ldg(t + 2 * (offset<LG>(P) + j)), b = __ldg(t + 2 * (offset<LG>(P) + j) + 1);
+    w1 = f2(a.x, a.y);
+    w2 = f2(a.z, a.w);
+    w4 = f2(b.x, b.y);
+    w8 = f2(b.z, b.w);
+  }
+};
+
 template <int LG, int DIR>
 struct RegFft {
   static constexpr int N = 1 << LG, TG = N >> 4;
@@ -131,13 +166,11 @@ struct RegFft {
   static constexpr int SMEM = N + (N >> 4);        // padded elements of the exchange array
   static_assert(LG >= 8, "at least two radix-16 passes");
 
-  // y_q *= W_L^{j q}, q = 1..15 (tw[k] = e^{-2 pi i k / TW}, k < TW / 2): four table
-  // values (j, 2j, 4j, 8j) and products of at most three of them
-  __device__ static void twiddle(float2 (&x)[16], int j, int lgL, const float2 *__restrict__ tw, int lgtw) {
-    const int s = j << (lgtw - lgL);
-    const bool cj = DIR > 0;
-    const float2 w1 = conj_if(__ldg(tw + s), cj), w2 = conj_if(__ldg(tw + 2 * s), cj);
-    const float2 w4 = conj_if(__ldg(tw + 4 * s), cj), w8 = conj_if(__ldg(tw + 8 * s), cj);
+  // y_q *= W_L^{j q}, q = 1..15: four table values (j, 2j, 4j, 8j) and products of at most three
+  // of them
+  template <int P, typename TW> __device__ static void twiddle(float2 (&x)[16], int j, TW tw) {
+    float2 w1, w2, w4, w8;
+    tw.template get<LG, P>(j, w1, w2, w4, w8);
     const float2 w3 = cmul(w1, w2), w5 = cmul(w1, w4), w6 = cmul(w2, w4), w7 = cmul(w3, w4);
     x[1] = cmul(x[1], w1);
     x[2] = cmul(x[2], w2);
@@ -156,8 +189,7 @@ struct RegFft {
     x[15] = cmul(x[15], cmul(w7, w8));
   }
 
-  template <int P>
-  __device__ static void pass(float2 (&x)[16], float2 *sm, int h, const float2 *__restrict__ tw, int lgtw) {
+  template <int P, typename TW> __device__ static void pass(float2 (&x)[16], float2 *sm, int h, TW tw) {
     constexpr bool R16 = P < NP16;
     constexpr int lgR = R16 ? 4 : (LG & 3);
     constexpr int R = 1 << lgR;
@@ -194,7 +226,7 @@ struct RegFft {
     if constexpr (!LAST) {
       static_assert(G == 1, "only the last pass may be shorter");
       const int j = h & (m - 1), Q = h >> lgm;
-      twiddle(x, j, lgL, tw, lgtw);
+      twiddle<P>(x, j, tw);
       if constexpr (P == 0) __syncthreads();  // the array's previous readers are done
       const int pb = rpad(Q * m + j);
       constexpr int st = S * m + ((S * m) >> 4);  // S m is a multiple of 16
@@ -217,12 +249,12 @@ struct RegFft {
   // The whole transform: x holds element h + TG c in slot c on entry and X[h + TG c]
   // on return; sm: SMEM elements (16-byte aligned) that only this group uses. Every
   // thread of the block must call it (it synchronises the block).
-  __device__ static void run(float2 (&x)[16], float2 *sm, int h, const float2 *__restrict__ tw, int lgtw) {
-    pass<0>(x, sm, h, tw, lgtw);
-    if constexpr (NPASS > 1) pass<1>(x, sm, h, tw, lgtw);
-    if constexpr (NPASS > 2) pass<2>(x, sm, h, tw, lgtw);
-    if constexpr (NPASS > 3) pass<3>(x, sm, h, tw, lgtw);
-    if constexpr (NPASS > 4) pass<4>(x, sm, h, tw, lgtw);
+  template <typename TW> __device__ static void run(float2 (&x)[16], float2 *sm, int h, TW tw) {
+    pass<0>(x, sm, h, tw);
+    if constexpr (NPASS > 1) pass<1>(x, sm, h, tw);
+    if constexpr (NPASS > 2) pass<2>(x, sm, h, tw);
+    if constexpr (NPASS > 3) pass<3>(x, sm, h, tw);
+    if constexpr (NPASS > 4) pass<4>(x, sm, h, tw);
     static_assert(NPASS <= 5, "up to 2^18");
   }
 };

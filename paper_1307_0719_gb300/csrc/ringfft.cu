@@ -129,7 +129,7 @@ __device__ __forceinline__ void reg_bluestein(float2 *Y, int SY, int ni, float2 
       float2 bq[16];
 #pragma unroll
       for (int c = 0; c < 16; ++c) bq[c] = __ldg(spec + hh + TGB * c);
-      Ff::run(x, xb, hh, tw, lgtw);
+      Ff::run(x, xb, hh, TwidTable<-1>{tw, lgtw});
 #pragma unroll
       for (int c = 0; c < 16; ++c) x[c] = cmul(x[c], bq[c]);
 #pragma unroll
@@ -137,17 +137,17 @@ __device__ __forceinline__ void reg_bluestein(float2 *Y, int SY, int ni, float2 
         const int pp = hh + TGB * c;
         bq[c] = pp < ni ? __ldg(chirp + pp) : f2(0.0f, 0.0f);
       }
-      Fi::run(x, xb, hh, tw, lgtw);
+      Fi::run(x, xb, hh, TwidTable<+1>{tw, lgtw});
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const int pp = hh + TGB * c;
         if (pp < ni) yq[pp] = cmul(x[c], bq[c]);
       }
     } else {
-      Ff::run(x, xb, hh, tw, lgtw);
+      Ff::run(x, xb, hh, TwidTable<-1>{tw, lgtw});
 #pragma unroll
       for (int c = 0; c < 16; ++c) x[c] = cmul(x[c], __ldg(spec + hh + TGB * c));
-      Fi::run(x, xb, hh, tw, lgtw);
+      Fi::run(x, xb, hh, TwidTable<+1>{tw, lgtw});
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const int pp = hh + TGB * c;

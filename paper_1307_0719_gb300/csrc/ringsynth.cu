@@ -25,11 +25,13 @@
 // ring's length the aliases are folded while staging (per map, since (m / L)^k is not a
 // function of m modulo the length).
 //
-// What bounds it: instruction issue (the belt kernel 61%, the cap kernels 67-70% issue-active at 24-32
-// warps per SM, DRAM under 30% of its peak). Sixteen T+Q/U realisations of order 4 take 135 ms at
-// Nside 2048 / lmax 3000 and 13.9 ms at Nside 512 / lmax 1024, against 232 and 21.9 ms for packed
-// pairs of maps with Bluestein's convolution in the caps (per map and pixel: 1.6 times the
-// instructions on the belt, 2 to 2.4 times in the caps).
+// What bounds it: instruction issue (the belt kernel 69%, the cap kernels 60-65% issue-active at 24-32
+// warps per SM, DRAM under 35% of its peak). Sixteen T+Q/U realisations of order 4 take 108 ms at
+// Nside 2048 / lmax 3000 and 10.8 ms at Nside 512 / lmax 1024, against 232 and 21.9 ms for packed
+// pairs of maps with Bluestein's convolution in the caps. Of this, one weight for a pixel and
+// its mirror image gave 6 ms at Nside 2048 (the cap kernels' instructions per map and pixel fell by
+// a fifth), and the packed twiddle table 19 ms (a warp's twiddle loads touched up to 88 lines
+// a pass, as much of the load path's time as all shared-memory traffic).
 #include <math.h>
 
 #include "regfft.cuh"
@@ -84,9 +86,18 @@ struct SyArgs {
   const float *rsinf;
   const int4 *rings;    // {ring, band, fold, mcut}
   const float2 *tw;     // e^{-2 pi i k / TW}, k < TW / 2
+  const float4 *tw4;    // twiddles of the passes of this length (TwidPacked)
   const float *corr;    // 1 / (window's transform) at m / (finest grid)
   int lgtw, mmax, rounds, chunks, rowcap;
   float invL;
+  long long tile;       // tile stride of the jobs whose output is tiled (the same for all of them)
+};
+
+// Output of one map of an interpolating CTA's round (out: null where there is none)
+struct __align__(16) SyOut {
+  float *out;
+  float scale;
+  int tiled;
 };
 
 // The aliases of class t (m = t + q N and m = q N - t) of one coefficient row with the
@@ -128,6 +139,7 @@ __global__ void __launch_bounds__(SyCfg<LG, MODE>::NT, SyCfg<LG, MODE>::CTAS)
   constexpr int H = C::H, TG = C::TG, NT = C::NT, N2 = 2 * H;
   constexpr bool INTERP = MODE != kSyDirect;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ SyOut outs[INTERP ? C::MAPS : 1];
   const int tid = threadIdx.x, g = tid / TG, h = tid - g * TG;
   const int ring = blockIdx.x / A.chunks, chunk = blockIdx.x - ring * A.chunks;
   const int4 R = A.rings[ring];
@@ -206,6 +218,17 @@ __global__ void __launch_bounds__(SyCfg<LG, MODE>::NT, SyCfg<LG, MODE>::CTAS)
       pk = k;
     }
     __syncthreads();
+    if (INTERP && tid < C::MAPS) {  // (every thread has left the round before)
+      const int ji = chunk * C::MAPS * A.rounds + tid * A.rounds + rd;
+      SyOut o = {nullptr, 0.0f, 0};
+      if (ji < jobs.n) {
+        const JobDev &J = jobs.job[ji];
+        o.out = (float *)J.out;
+        o.scale = J.scalef * (J.div_sint ? rs : 1.0f);
+        o.tiled = J.tile != 0;
+      }
+      outs[tid] = o;
+    }
     float2 x[16];
     {
       const float2 wh = conj_if(__ldg(A.tw + (h << (A.lgtw - LG - 1))), true);  // e^{2 pi i h / 2H}
@@ -230,13 +253,20 @@ __global__ void __launch_bounds__(SyCfg<LG, MODE>::NT, SyCfg<LG, MODE>::CTAS)
         x[0] = f2(s0 + sH, s0 - sH);
       }
     }
-    F::run(x, xb, h, A.tw, A.lgtw);
+    F::run(x, xb, h, TwidPacked{A.tw4});
     if (!INTERP) {
       if (act) {
         const JobDev &J = jobs.job[jid];
         const float sc = J.scalef * (J.div_sint ? rs : 1.0f);
         float *out = (float *)J.out;
-        if (N == N2) {
+        if (N == N2 && 2 * TG >= kD3Tile) {
+          // slots lie a multiple of the tile's pixels apart: a constant distance in either layout
+          const long long p = first + 2 * h;
+          float *o = out + (J.tile ? d3_pix(p, J.tile) : p);
+          const long long step = J.tile ? (long long)(2 * TG / kD3Tile) * J.tile : 2 * TG;
+#pragma unroll
+          for (int c = 0; c < 16; ++c) *(float2 *)(o + c * step) = f2(sc * x[c].x, sc * x[c].y);
+        } else if (N == N2) {
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
             const long long p = first + 2 * (h + TG * c);
@@ -276,11 +306,11 @@ __global__ void __launch_bounds__(SyCfg<LG, MODE>::NT, SyCfg<LG, MODE>::CTAS)
       const int den = 2 * N;
       const float inv = 1.0f / (float)den, inv2 = 0.5f * inv;
       const float *g0 = (const float *)xch + 8;
-      const int sh = shifted ? 1 : 0;
-      const int jb = chunk * C::MAPS * A.rounds + rd;  // job of map 0 of this round; map i: + i rounds
-      for (int p = tid; p < N; p += NT) {
-        // position on the fine grid: (2 p + sh) 2^NFL / (2 N) = i0 + rem / den
-        const int num = (2 * p + sh) << NFL;
+      // Pixel p of a half-pixel-shifted ring (every cap ring) sits at (2 p + 1) 2^NFL / (2 N) = i0 +
+      // rem / den on the fine grid, and pixel N - 1 - p at its mirror image: the same weights, in
+      // reverse, serve both, for all maps of the round
+      for (int p = tid; p < N / 2; p += NT) {
+        const int num = (2 * p + 1) << NFL;
         int i0 = (int)((float)num * inv);
         int rem = num - i0 * den;
         if (rem < 0) {
@@ -308,34 +338,37 @@ __global__ void __launch_bounds__(SyCfg<LG, MODE>::NT, SyCfg<LG, MODE>::CTAS)
           wt[t] = fmaf(s, o, e);
           wt[W - 1 - t] = fmaf(-s, o, e);
         }
-        const long long gp = first + p;
-        const int b0 = i0 - HW + 1;  // the first of the W points
-        if (MODE == kSyTwice) {
-          // fine point f is point f >> 1 of grid f & 1
-          const float *ga = g0 + (b0 & 1) * (2 * C::X) + (b0 >> 1);
-          const float *gb = g0 + ((b0 & 1) ^ 1) * (2 * C::X) + ((b0 + 1) >> 1);
-          float acc = 0.0f;
+        const int b0 = i0 - HW + 1, b1 = (1 << NFL) - i0 - HW;  // the first of the W points of either pixel
+        const long long pa = first + p, pb = first + N - 1 - p;
+        const long long ta = d3_pix(pa, A.tile), tb = d3_pix(pb, A.tile);
 #pragma unroll
-          for (int t = 0; t < HW; ++t) {
-            acc = fmaf(wt[2 * t], ga[t], acc);
-            acc = fmaf(wt[2 * t + 1], gb[t], acc);
-          }
-          if (jb < jobs.n) {
-            const JobDev &J = jobs.job[jb];
-            ((float *)J.out)[J.tile ? d3_pix(gp, J.tile) : gp] = acc * (J.scalef * (J.div_sint ? rs : 1.0f));
-          }
-        } else {
+        for (int i = 0; i < C::MAPS; ++i) {
+          const SyOut o = outs[i];
+          if (!o.out) break;  // (the maps of a round are its first ones)
+          float va = 0.0f, vb = 0.0f;
+          if (MODE == kSyTwice) {
+            // fine point f is point f >> 1 of grid f & 1
+            const float *a0 = g0 + (b0 & 1) * (2 * C::X) + (b0 >> 1);
+            const float *a1 = g0 + ((b0 & 1) ^ 1) * (2 * C::X) + ((b0 + 1) >> 1);
+            const float *c0 = g0 + (b1 & 1) * (2 * C::X) + (b1 >> 1);
+            const float *c1 = g0 + ((b1 & 1) ^ 1) * (2 * C::X) + ((b1 + 1) >> 1);
 #pragma unroll
-          for (int i = 0; i < C::MAPS; ++i) {
-            const int ji = jb + i * A.rounds;
-            if (ji >= jobs.n) break;
-            const float *gi = g0 + i * (2 * C::X) + b0;
-            float acc = 0.0f;
+            for (int t = 0; t < HW; ++t) {
+              va = fmaf(wt[2 * t], a0[t], va);
+              va = fmaf(wt[2 * t + 1], a1[t], va);
+              vb = fmaf(wt[W - 1 - 2 * t], c0[t], vb);
+              vb = fmaf(wt[W - 2 - 2 * t], c1[t], vb);
+            }
+          } else {
+            const float *gi = g0 + i * (2 * C::X);
 #pragma unroll
-            for (int t = 0; t < W; ++t) acc = fmaf(wt[t], gi[t], acc);
-            const JobDev &J = jobs.job[ji];
-            ((float *)J.out)[J.tile ? d3_pix(gp, J.tile) : gp] = acc * (J.scalef * (J.div_sint ? rs : 1.0f));
+            for (int t = 0; t < W; ++t) {
+              va = fmaf(wt[t], gi[b0 + t], va);
+              vb = fmaf(wt[W - 1 - t], gi[b1 + t], vb);
+            }
           }
+          o.out[o.tiled ? ta : pa] = va * o.scale;
+          o.out[o.tiled ? tb : pb] = vb * o.scale;
         }
       }
       // the next round's first pass stores to the exchange arrays behind a barrier
@@ -430,6 +463,31 @@ const float *host_synth_window(SyWindow *w) {
   return s.corr;
 }
 
+// Twiddles of the transforms of length 2^8 .. 2^12 (TwidPacked), one length after another
+static constexpr int synth_twiddle_offset(int lg) {
+  int n = 0;
+  for (int g = 8; g < lg; ++g)
+    for (int p = 0; 4 * p + 4 <= g; ++p) n += 1 << (g - 4 * p - 4);
+  return n;
+}
+int host_synth_twiddles(float *out) {
+  const int n = synth_twiddle_offset(13);
+  if (!out) return n;
+  for (int g = 8; g <= 12; ++g) {
+    float *o = out + 8 * (size_t)synth_twiddle_offset(g);
+    for (int p = 0; 4 * p + 4 <= g; ++p) {
+      const int L = 1 << (g - 4 * p);
+      for (int j = 0; j < L / 16; ++j, o += 8)
+        for (int q = 0; q < 4; ++q) {
+          const double a = 2.0 * M_PI * (double)(j << q) / (double)L;
+          o[2 * q] = (float)cos(a);
+          o[2 * q + 1] = (float)sin(a);
+        }
+    }
+  }
+  return n;
+}
+
 // Group of one ring, by its length and band (mcut: its coefficients beyond are zero):
 // the belt on its own grid; the caps on the smallest grid that oversamples their band,
 // which is half the ring's length where folding the aliases buys a smaller grid.
@@ -503,11 +561,18 @@ static cudaError_t synth_launch(const tl_plan *p, const SyGroup &g, const JobLis
   A.rsinf = p->ring.rsinf;
   A.rings = p->sy_rings + g.first;
   A.tw = (const float2 *)p->twiddle;
+  A.tw4 = p->sy_tw4 + 2 * synth_twiddle_offset(LG);
   A.corr = MODE == kSyTwice ? p->sy_corr + kSyCorr : p->sy_corr;
   A.lgtw = 31 - __builtin_clz((unsigned)p->tw_len);
   A.mmax = p->mmax;
   A.rowcap = (g.band + 2) & ~1;
   A.invL = (float)(1.0 / (double)(p->lmax + 1));
+  A.tile = 0;
+  for (int i = 0; i < jl.n; ++i)
+    if (jl.job[i].tile) {
+      if (A.tile && A.tile != jl.job[i].tile) return cudaErrorInvalidValue;
+      A.tile = jl.job[i].tile;
+    }
   // jobs of a CTA: its groups take `rounds` consecutive jobs each (one plane's maps
   // follow one another, so a row is staged about once per plane and ring), short enough that the
   // launch has about sixteen CTAs per resident one
