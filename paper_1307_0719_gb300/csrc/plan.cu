@@ -402,16 +402,15 @@ extern "C" long long tl_plan_batch_launches(const tl_plan *p, int nreal, int wit
     // per batch: coefficient tiles and Legendre launch of T, the potential and Q/U
     const long long chunks = (nreal + p->batch - 1) / p->batch;
     const long long per_chunk = 2 + (phi ? 2 : 0) + (pol ? 2 : 0);
-    // per realisation: deflection FFT, derivative-map FFT, gather and its double pass
-    return chunks * per_chunk + (long long)nreal * ((phi ? G : 0) + G + 2 + sub);
+    // per realisation: ring FFTs (deflection and derivative maps together), gather and its double pass
+    return chunks * per_chunk + (long long)nreal * (G + 2 + sub);
   }
   const bool fuse = phi && p->order >= 1;
   long long per = 0;
   if (phi && !fuse) per += 2 + G;  // stand-alone deflection: prep, Legendre, FFT
   per += 2 + (fuse ? 1 : 0);       // spin-0 prep (T, and phi when fused), Legendre
-  if (fuse) per += G;              // deflection FFT
   if (pol) per += 2;               // spin-2 prep, Legendre
-  per += G + (p->precision == TL_FP64 ? 1 : 2);  // derivative-map FFT, gather (float: and its double pass)
+  per += G + (p->precision == TL_FP64 ? 1 : 2);  // ring FFTs (with a fused deflection's), gather (float: and its double pass)
   return (long long)nreal * (per + sub);
 }
 
@@ -422,20 +421,22 @@ static void mark(tl_plan *p, int i, cudaStream_t s) {
   if (p->timing && i < 8) cudaEventRecord(p->ev[i], s);
 }
 
-// alpha from the phi planes (j = 0, 1) already in d7_P
+// the jobs of alpha from the phi planes (j = 0, 1)
 // il: the phi planes come from the tensor-core stage (four-ring interleaved rows)
-static tl_status deflection_fft(tl_plan *p, void *ath, void *aph, cudaStream_t s, int il = 0) {
+static void deflection_jobs(const tl_plan *p, void *ath, void *aph, int il, MapJob *jobs) {
   const double L = deriv_norm(p);
-  MapJob jobs[2] = {{3, 1, 0, 0, L, ath, 0, il}, {3, 0, 1, 1, L, aph, 0, il}};
-  TRY_CUDA(launch_ringfft(p, jobs, 2, 2, s));
-  return TL_OK;
+  jobs[0] = MapJob{3, 1, 0, 0, L, ath, 0, il};
+  jobs[1] = MapJob{3, 0, 1, 1, L, aph, 0, il};
 }
 
 // stand-alone deflection: phi through the spin-0 stage alone (uses rec_T)
 static tl_status deflection_impl(tl_plan *p, const double *alm_phi, void *ath, void *aph, cudaStream_t s) {
   TRY_CUDA(launch_prep_spin0(p, alm_phi, nullptr, s));
   TRY_CUDA(launch_legendre_spin0(p, 1, false, p->d7_P, nullptr, s));
-  return deflection_fft(p, ath, aph, s);
+  MapJob jobs[2];
+  deflection_jobs(p, ath, aph, 0, jobs);
+  TRY_CUDA(launch_ringfft(p, jobs, 2, 2, s));
+  return TL_OK;
 }
 
 // the plan's deflection: on its own plan at lmax_phi when one is set
@@ -542,10 +543,15 @@ extern "C" tl_status tl_synth_derivs(tl_plan *p, const double *alm, int spin, vo
   return TL_OK;
 }
 
-// ring FFTs into Taylor-ready maps d_th^j d_ph^k s / (j! k! L^(j+k)) for one realisation
-static tl_status lens_fft(tl_plan *p, const void *const *planes, cudaStream_t s, int il) {
+// ring FFTs into Taylor-ready maps d_th^j d_ph^k s / (j! k! L^(j+k)) for one realisation, and with
+// phi into the deflection (from the phi planes) in the same launches
+static tl_status lens_fft(tl_plan *p, const void *const *planes, bool phi, cudaStream_t s, int il) {
   const bool pol = (p->spins & TL_SPIN_QU) != 0;
   std::vector<MapJob> jobs;
+  if (phi) {  // a pair of its own
+    jobs.resize(2);
+    deflection_jobs(p, p->alpha, (char *)p->alpha + (size_t)p->elem * p->npix, il, jobs.data());
+  }
   // Jobs are packed two per transform in list order. Q and U of the same (j, k)
   // pair (similar magnitudes) and come first, an even count; then the T maps, which
   // pair within one coefficient plane j (the fold reads the row once for both),
@@ -584,17 +590,13 @@ tl_status lens_stage_after_legendre(tl_plan *p, int nreal, bool phi, void *const
       const size_t off = (size_t)r * p->d7_rstride * t2, offp = (size_t)r * p->d7p_rstride * t2;
       const void *planes[4] = {(char *)p->d7_T + off, pol ? (char *)p->d7_Q + off : nullptr,
                                pol ? (char *)p->d7_U + off : nullptr, (char *)p->d7_P + offp};
-      if (phi) {
-        const double L = deriv_norm(p);
-        MapJob jobs[2] = {{3, 1, 0, 0, L, ath, 0, 1}, {3, 0, 1, 1, L, aph, 0, 1}};
-        TRY_CUDA(launch_ringfft_planes(p, planes, jobs, 2, s));
-      } else if (aP && aP[r] && p->phi_plan) {
+      if (!phi && aP && aP[r] && p->phi_plan) {
         tl_status st = plan_deflection(p, aP[r], ath, aph, s);
         if (st != TL_OK) return st;
-      } else {
+      } else if (!phi) {
         TRY_CUDA(cudaMemsetAsync(p->alpha, 0, 2 * mapb, s));
       }
-      tl_status st = lens_fft(p, planes, s, 1);
+      tl_status st = lens_fft(p, planes, phi, s, 1);
       if (st != TL_OK) return st;
       if (tm) cudaEventRecord(p->evr[3 * r + 1], s);
       TRY_CUDA(launch_gather(p, p->alpha, p->d3, To[r], pol ? Qo[r] : nullptr, pol ? Uo[r] : nullptr, s));
@@ -666,13 +668,8 @@ static tl_status lens_chunk(tl_plan *p, int nreal, const double *const *aT, cons
   mark(p, 1, s);
   TRY_CUDA(launch_legendre_spin0(p, p->order, fuse, p->d7_T, p->d7_P, s));
   mark(p, 2, s);
-  // 2. deflection alpha = grad phi at the pixel centres
-  if (fuse) {
-    tl_status st = deflection_fft(p, ath, aph, s);
-    if (st != TL_OK) return st;
-  } else if (!alm_phi) {
-    TRY_CUDA(cudaMemsetAsync(p->alpha, 0, 2 * mapb, s));
-  }
+  // 2. deflection alpha = grad phi at the pixel centres: with the ring FFTs below
+  if (!alm_phi) TRY_CUDA(cudaMemsetAsync(p->alpha, 0, 2 * mapb, s));
   mark(p, 3, s);
   // 3. spin-2 Legendre stage
   if (pol) TRY_CUDA(launch_prep_spin2(p, alm_E, alm_B, s));
@@ -681,7 +678,7 @@ static tl_status lens_chunk(tl_plan *p, int nreal, const double *const *aT, cons
   mark(p, 5, s);
   // 4. ring FFTs
   const void *planes[4] = {p->d7_T, p->d7_Q, p->d7_U, p->d7_P};
-  tl_status st = lens_fft(p, planes, s, 0);
+  tl_status st = lens_fft(p, planes, fuse, s, 0);
   if (st != TL_OK) return st;
   mark(p, 6, s);
   // 5. gather + Taylor + rotate
@@ -767,14 +764,9 @@ static tl_status forward_derivs(tl_plan *p, const double *alm_T, const double *a
   }
   // the tensor-core stage leaves its planes four-ring interleaved
   const int il = p->batch > 1 ? 1 : 0;
-  if (alm_phi && !defl_done) {
-    tl_status st = deflection_fft(p, ath, aph, s, il);
-    if (st != TL_OK) return st;
-  } else if (!alm_phi) {
-    TRY_CUDA(cudaMemsetAsync(p->alpha, 0, 2 * mapb, s));
-  }
+  if (!alm_phi) TRY_CUDA(cudaMemsetAsync(p->alpha, 0, 2 * mapb, s));
   const void *planes[4] = {p->d7_T, p->d7_Q, p->d7_U, p->d7_P};
-  return lens_fft(p, planes, s, il);
+  return lens_fft(p, planes, alm_phi && !defl_done, s, il);
 }
 
 extern "C" tl_status tl_lens_adjoint(tl_plan *p, const double *alm_T, const double *alm_E, const double *alm_B,

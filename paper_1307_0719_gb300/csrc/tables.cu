@@ -136,8 +136,8 @@ long long host_bluestein_layout(int nside, long long *off, int *ml, int *maxm) {
 }
 
 // Rings of each ring-FFT launch: the equatorial belt, then the caps by Bluestein
-// length M (largest first), then the power-of-two caps; each group's rings are
-// ordered by decreasing length. No allocation.
+// length M (largest first), then the power-of-two caps (up to Nside 256: all power-of-two
+// rings, then all Bluestein rings); each kind's rings are ordered by decreasing length. No allocation.
 int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGroup *groups, int *order,
                     const unsigned char *use) {
   int ng = 0, n = 0;
@@ -160,10 +160,32 @@ int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGr
     ++ng;
     return true;
   };
+  // Small spheres: one launch for all power-of-two rings and one for all Bluestein rings, whatever
+  // their lengths (the kernels take a ring's own). Their groups would each be a launch of a few blocks
+  // bound by latency, one after another; from Nside 512 on a group fills the chip, and the
+  // shared memory of the longest ring would keep blocks of short ones out.
+  const bool few = nside <= 256;
+  auto merge = [&](int from) {
+    for (int i = from + 1; i < ng; ++i) {
+      FftGroup &a = groups[from];
+      const FftGroup &b = groups[i];
+      a.count += b.count;
+      if (b.ni_max > a.ni_max) a.ni_max = b.ni_max;
+      if (b.ni_min < a.ni_min) a.ni_min = b.ni_min;
+      if (b.M > a.M) a.M = b.M;
+    }
+    if (ng > from) ng = from + 1;
+  };
   if (!add(-1)) return -1;
+  if (few) {
+    if (!add(0)) return -1;
+    merge(0);
+  }
+  const int blue = ng;
   for (int M = 1 << 30; M >= 2; M >>= 1)
     if (M <= 4 * nside && !add(M)) return -1;
-  if (!add(0)) return -1;
+  if (few) merge(blue);
+  else if (!add(0)) return -1;
   int want = nrings;
   if (use) {
     want = 0;
@@ -192,8 +214,16 @@ void host_ring_bands(int nside, int lmax, int h, const double *sint, const doubl
       if (a >= 1.0 || b >= 1.0) return 1e9;
       return m * atanh(a) - L * atanh(b);
     };
-    int lo = 0, hi = lmax;
-    if (damp(lmax) < most) {
+    // the cut grows from the pole to the equator: gallop on from the ring before
+    int lo = r > 0 ? mcut[r - 1] : 0, hi = lmax, step = 1;
+    if (lo > 3) lo -= 3;
+    if (damp(lo) >= most) lo = 0;
+    while (lo + step < lmax && damp(lo + step) < most) {
+      lo += step;
+      step *= 2;
+    }
+    if (lo + step < lmax) hi = lo + step;
+    if (hi == lmax && damp(lmax) < most) {
       lo = lmax;
     } else {
       while (hi - lo > 1) {
