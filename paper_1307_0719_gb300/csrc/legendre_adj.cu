@@ -324,6 +324,281 @@ __global__ void __launch_bounds__(128) legendre_adj2_kernel(RingTable rt, const 
                                 live);
 }
 
+// ---------------------------------------------------------------------------
+// The same in single precision, with the instructions per step near the arithmetic's own (as in
+// legendre_f32.cu): the step factors of a window are staged in shared memory, the steps run without the
+// tests of the scale once every ring of the warp has reached 0, and the parity of l + m is that
+// of the position in the window (the spin-2 sums U1 and U2 change places once, at m = 1, instead of
+// being selected in every step). Every value is formed by the same operations in the same order.
+// Order 4, Nside 1024 / lmax 2048: spin 2 25.7 -> 16.6 ms, spin 0 with the potential 9.7 -> 7.8 ms (101 ->
+// about 62 instructions per ring and step at spin 2); at order 0, the whole analysis, 23.6 -> 14.2 ms.
+
+template <int NDER, bool PHI>
+__global__ void __launch_bounds__(128) legendre_adj0_f32_kernel(RingTable rt, const double *__restrict__ lnorm0,
+                                                                int nside, int lmax, int mmax, int nrings,
+                                                                const int *__restrict__ mcut, int nder_T,
+                                                                const float2 *__restrict__ tab,
+                                                                const float2 *__restrict__ FT,
+                                                                const float2 *__restrict__ FP,
+                                                                double *__restrict__ accT, double *__restrict__ accP) {
+  constexpr int NT = 128, WV = AdjWin<float>::WV, V = PHI ? 4 : 2, W = WV / V;
+  __shared__ float win[NT][WV + 1];
+  __shared__ float2 aq[2][W];  // A, Q
+  const int m = blockIdx.y;
+  const int tid = threadIdx.x;
+  const int rn = blockIdx.x * NT + tid;
+  const bool active = rn < 2 * nside && m <= mmax;
+  const int r = active ? rn : 0;
+  // a block none of whose rings leaves zero at this m (host_ring_bands) adds nothing; a warp of
+  // such rings runs no steps
+  const bool live = __any_sync(0xffffffffu, active && (!mcut || m <= mcut[r]));
+  if (!__syncthreads_or(live)) return;
+  const int rs = nrings - 1 - r;
+  const double invL = 1.0 / (double)(lmax + 1);
+  const size_t ld = (size_t)(mmax + 1);
+  const int mm = m <= mmax ? m : mmax;
+
+  // [parity of l - m][j]: G+ and G- (see legendre_adj0_kernel)
+  float gr[2][NDER + 1], gi[2][NDER + 1], hr[2][2], hi[2][2];
+#pragma unroll
+  for (int j = 0; j <= NDER; ++j) {
+    float2 fn = {0.0f, 0.0f}, fs = {0.0f, 0.0f};
+    if (active && j <= nder_T) {
+      fn = FT[((size_t)j * nrings + r) * ld + mm];
+      if (rs != r) fs = FT[((size_t)j * nrings + rs) * ld + mm];
+    }
+    const float sg = (j & 1) ? -1.0f : 1.0f;
+    gr[0][j] = fn.x + sg * fs.x;
+    gi[0][j] = fn.y + sg * fs.y;
+    gr[1][j] = fn.x - sg * fs.x;
+    gi[1][j] = fn.y - sg * fs.y;
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    float2 fn = {0.0f, 0.0f}, fs = {0.0f, 0.0f};
+    if (PHI && active) {
+      fn = FP[((size_t)j * nrings + r) * ld + mm];
+      if (rs != r) fs = FP[((size_t)j * nrings + rs) * ld + mm];
+    }
+    const float sg = (j & 1) ? -1.0f : 1.0f;
+    hr[0][j] = fn.x + sg * fs.x;
+    hi[0][j] = fn.y + sg * fs.y;
+    hr[1][j] = fn.x - sg * fs.x;
+    hi[1][j] = fn.y - sg * fs.y;
+  }
+  Leib<float, NDER> LC;
+  leibniz_coefs<float, NDER>(rt.z[r], rt.sint[r], invL, LC);
+  float d[NDER + 1], v[NDER + 1];
+  int sc;
+  seed_spin0<float, NDER>(rt, lnorm0, r, m, invL, v, sc);
+  rec_init<float, NDER>(d, v);
+  const float w = (float)rt.omza[r];
+  const long long base = (long long)m * (2 * lmax + 1 - m) / 2;
+  auto load = [&](int lb, int buf) {
+    if (tid < W && lb + tid <= lmax) {
+      const float Q = __ldg(&tab[base + lb + tid].y);
+      aq[buf][tid] = make_float2(2.0f + Q, Q);
+    }
+  };
+  float *row = win[tid];
+  if (!live)
+    for (int i = 0; i < WV; ++i) row[i] = 0.0f;
+  bool plain = false;  // every ring of the warp at scale 0
+  load(m, 0);
+  __syncthreads();
+  int buf = 0;
+  for (int lb = m; lb <= lmax; lb += W, buf ^= 1) {
+    const int n = min(W, lmax - lb + 1);
+    // l - m and the position i have one parity (W is even)
+    auto sums = [&](int i, int p, bool on) {
+      float cr = 0.0f, ci = 0.0f, pr = 0.0f, pi = 0.0f;
+      if (on) {
+#pragma unroll
+        for (int j = 0; j <= NDER; ++j) {
+          cr = fmaf(v[j], gr[p][j], cr);
+          ci = fmaf(v[j], gi[p][j], ci);
+        }
+        if (PHI) {
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            pr = fmaf(v[j], hr[p][j], pr);
+            pi = fmaf(v[j], hi[p][j], pi);
+          }
+        }
+      }
+      row[i * V + 0] = cr;
+      row[i * V + 1] = ci;
+      if (PHI) {
+        row[i * V + 2] = pr;
+        row[i * V + 3] = pi;
+      }
+    };
+    if (live) {
+      int i = 0;
+#pragma unroll 1
+      for (; i < n && !plain; i += 2) {
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          if (i + p >= n) break;
+          const float2 f = aq[buf][i + p];
+          sums(i + p, p, sc == 0);
+          step_diff<float, NDER, 1>(v, d, LC, w, f.x, f.y);
+          rescale<float, NDER>(d, v, v[0], sc);
+        }
+        plain = __all_sync(0xffffffffu, sc == 0);  // and stays so
+      }
+#pragma unroll 2
+      for (; i + 1 < n; i += 2) {
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          const float2 f = aq[buf][i + p];
+          sums(i + p, p, true);
+          step_diff<float, NDER, 1>(v, d, LC, w, f.x, f.y);
+        }
+      }
+      if (i < n) sums(i, 0, true);  // l = lmax
+    }
+    load(lb + W, buf ^ 1);
+    flush_window<float, NT, WV, V>(win, n, base + lb, accT, PHI ? accP : nullptr);
+  }
+}
+
+// a warp's steps through one window: U1 = (u1r, u1i) at even positions, U2 at odd ones
+template <int NDER, int SG>
+__device__ __forceinline__ void adj2_window(const float2 *__restrict__ aq, int n, bool &plain,
+                                            const Leib<float, NDER> &LC, float w, float (&v)[NDER + 1],
+                                            float (&d)[NDER + 1], int &sc, const float (&ur)[2][NDER + 1],
+                                            const float (&ui)[2][NDER + 1], float *__restrict__ row) {
+  auto sums = [&](int i, int p, bool on) {
+    float er = 0.0f, ei = 0.0f, fr = 0.0f, fi = 0.0f;
+    if (on) {
+#pragma unroll
+      for (int j = 0; j <= NDER; ++j) {
+        er = fmaf(v[j], ur[p][j], er);
+        ei = fmaf(v[j], ui[p][j], ei);
+        fr = fmaf(v[j], ur[p ^ 1][j], fr);
+        fi = fmaf(v[j], ui[p ^ 1][j], fi);
+      }
+    }
+    row[i * 4 + 0] = er;
+    row[i * 4 + 1] = ei;
+    row[i * 4 + 2] = fr;
+    row[i * 4 + 3] = fi;
+  };
+  int i = 0;
+#pragma unroll 1
+  for (; i < n && !plain; i += 2) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      if (i + p >= n) break;
+      const float2 f = aq[i + p];
+      sums(i + p, p, sc == 0);
+      step_diff<float, NDER, SG>(v, d, LC, w, f.x, f.y);
+      rescale<float, NDER>(d, v, v[0], sc);
+    }
+    plain = __all_sync(0xffffffffu, sc == 0);  // and stays so
+  }
+#pragma unroll 2
+  for (; i + 1 < n; i += 2) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const float2 f = aq[i + p];
+      sums(i + p, p, true);
+      step_diff<float, NDER, SG>(v, d, LC, w, f.x, f.y);
+    }
+  }
+  if (i < n) sums(i, 0, true);  // l = lmax
+}
+
+template <int NDER>
+__global__ void __launch_bounds__(128) legendre_adj2_f32_kernel(RingTable rt, const double *__restrict__ lnorm0,
+                                                                int nside, int lmax, int mmax, int nrings,
+                                                                const int *__restrict__ mcut,
+                                                                const Rec2<float> *__restrict__ rec,
+                                                                const float2 *__restrict__ FQ,
+                                                                const float2 *__restrict__ FU,
+                                                                double *__restrict__ accE, double *__restrict__ accB) {
+  constexpr int NT = 128, RP = 64, WV = AdjWin<float>::WV, V = 4, W = WV / V;
+  __shared__ float win[NT][WV + 1];
+  __shared__ float2 aq[2][2][W];  // [buffer][north, mirror] A, Q
+  const int m = blockIdx.y;
+  const int t = threadIdx.x;
+  const int rn = blockIdx.x * RP + (t % RP);
+  const bool mirror = t >= RP;
+  const bool equator = rn == nrings - 1 - rn;
+  // the equator ring is its own mirror: its north thread carries both terms
+  const bool active = rn < 2 * nside && m <= mmax && !(mirror && equator);
+  const int r = rn < 2 * nside ? (mirror ? nrings - 1 - rn : rn) : 0;
+  const int rp = nrings - 1 - r;  // partner (mirror) ring
+  // (as for spin 0)
+  const bool live = __any_sync(0xffffffffu, active && (!mcut || m <= mcut[r]));
+  if (!__syncthreads_or(live)) return;
+  const double invL = 1.0 / (double)(lmax + 1);
+  const size_t ld = (size_t)(mmax + 1);
+  const int mm = m <= mmax ? m : mmax;
+  const int l0 = m > 2 ? m : 2;
+  const int par0 = (l0 + m) & 1;  // parity of l + m at l0 (1 at m = 1 only)
+
+  // [0]: U1 = S1bar + S2bar (even l + m), [1]: U2 = S1bar - S2bar (odd), or the other way round
+  // where l0 + m is odd
+  float ur[2][NDER + 1], ui[2][NDER + 1];
+#pragma unroll
+  for (int j = 0; j <= NDER; ++j) {
+    float2 q = {0.0f, 0.0f}, u = {0.0f, 0.0f}, qp = {0.0f, 0.0f}, up = {0.0f, 0.0f};
+    if (active) {
+      q = FQ[((size_t)j * nrings + r) * ld + mm];
+      u = FU[((size_t)j * nrings + r) * ld + mm];
+      qp = FQ[((size_t)j * nrings + rp) * ld + mm];
+      up = FU[((size_t)j * nrings + rp) * ld + mm];
+    }
+    const float h = 0.5f, sg = (j & 1) ? -0.5f : 0.5f;
+    // S1bar = -(q + i u)/2
+    const float s1r = -h * (q.x - u.y), s1i = -h * (q.y + u.x);
+    // S2bar = (-1)^j (-qp + i up)/2
+    const float s2r = sg * (-qp.x - up.y), s2i = sg * (-qp.y + up.x);
+    const float ar = s1r + s2r, ai = s1i + s2i, br = s1r - s2r, bi = s1i - s2i;
+    ur[0][j] = par0 ? br : ar;
+    ui[0][j] = par0 ? bi : ai;
+    ur[1][j] = par0 ? ar : br;
+    ui[1][j] = par0 ? ai : bi;
+  }
+  Leib<float, NDER> LC;
+  leibniz_coefs<float, NDER>(rt.z[r], rt.sint[r], invL, LC);
+  float d[NDER + 1], v[NDER + 1];
+  int sc;
+  (void)seed_spin2<float, NDER>(rt, lnorm0, r, m, invL, v, sc);
+  rec_init<float, NDER>(d, v);
+  if (l0 > lmax) return;  // uniform over the block
+  const float w = (float)rt.omza[r];
+  const long long base = (long long)m * (2 * lmax + 1 - m) / 2;
+  const Rec2<float> *rm = rec + base;
+  auto load = [&](int lb, int buf) {
+    if (t < W && lb + t <= lmax) {
+      const float4 f = __ldg((const float4 *)(rm + lb + t) + 1);  // A, m s / (l (l + 1)), Qn, Qs
+      aq[buf][0][t] = make_float2(f.x, f.z);
+      aq[buf][1][t] = make_float2(f.x, f.w);
+    }
+  };
+  float *row = win[t];
+  if (!live)
+    for (int i = 0; i < WV; ++i) row[i] = 0.0f;
+  bool plain = false;  // every ring of the warp at scale 0
+  load(l0, 0);
+  __syncthreads();
+  int buf = 0;
+  for (int lb = l0; lb <= lmax; lb += W, buf ^= 1) {
+    const int n = min(W, lmax - lb + 1);
+    if (live) {  // mirror threads (cos th < 0) are warps 2 and 3
+      if (mirror)
+        adj2_window<NDER, -1>(aq[buf][1], n, plain, LC, w, v, d, sc, ur, ui, row);
+      else
+        adj2_window<NDER, 1>(aq[buf][0], n, plain, LC, w, v, d, sc, ur, ui, row);
+    }
+    load(lb + W, buf ^ 1);
+    flush_window<float, NT, WV, V>(win, n, base + lb, accE, accB);
+  }
+}
+
 // Final scaling: abar = k_l acc; B's accumulator holds f with Bbar = -i k f;
 // m = 0 coefficients are real in the forward map, so their imaginary gradient is 0.
 template <typename T>
@@ -365,7 +640,12 @@ static cudaError_t adj0(const tl_plan *p, int nder_T, const void *FT, const void
                         cudaStream_t s) {
   typedef typename RealTraits<T>::T2 T2;
   dim3 grid((2 * p->nside + 127) / 128, p->mmax + 1);
-  legendre_adj0_kernel<T, NDER, PHI><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax,
+  if constexpr (sizeof(T) == 4)
+    legendre_adj0_f32_kernel<NDER, PHI><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax,
+                                                             p->nrings, p->mcut, nder_T, (const T2 *)p->tab0,
+                                                             (const T2 *)FT, (const T2 *)FP, aT, aP);
+  else
+    legendre_adj0_kernel<T, NDER, PHI><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax,
                                                           p->nrings, p->mcut, nder_T, (const T2 *)p->tab0, (const T2 *)FT,
                                                           (const T2 *)FP, aT, aP);
   return cudaGetLastError();
@@ -401,7 +681,12 @@ template <typename T, int NDER>
 static cudaError_t adj2(const tl_plan *p, const void *FQ, const void *FU, double *aE, double *aB, cudaStream_t s) {
   typedef typename RealTraits<T>::T2 T2;
   dim3 grid((2 * p->nside + 63) / 64, p->mmax + 1);
-  legendre_adj2_kernel<T, NDER><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings, p->mcut,
+  if constexpr (sizeof(T) == 4)
+    legendre_adj2_f32_kernel<NDER><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings,
+                                                        p->mcut, (const Rec2<float> *)p->rec_QU, (const T2 *)FQ,
+                                                        (const T2 *)FU, aE, aB);
+  else
+    legendre_adj2_kernel<T, NDER><<<grid, 128, 0, s>>>(p->ring, p->lnorm0, p->nside, p->lmax, p->mmax, p->nrings, p->mcut,
                                                      (const Rec2<T> *)p->rec_QU, (const T2 *)FQ, (const T2 *)FU, aE,
                                                      aB);
   return cudaGetLastError();
