@@ -866,6 +866,26 @@ __global__ void __launch_bounds__(umma_threads(Tc0<NDER, MODE, CNC>::NH), (Tc0<N
   umma_close<TM::cols, TM::NB, C::NH>(D, U);
 }
 
+// One unit of the persistent kernel, as a function of its own: inlined three times into the item
+// loop, the units' compute warps spilled 600 bytes. Barriers are fresh (counts start at 0).
+// Returns the state that umma_close needs.
+template <int NDER, int MODE, int NC, int NB, int NH, bool SPIN2>
+__device__ __noinline__ uint4 unit_call(const TcDesc *desc, int m, int rblk, unsigned char *sm, uint32_t tmem,
+                                        uint32_t bars, volatile int *abort) {
+  const TcDesc D = *desc;
+  UmmaCta U;
+  U.tmem = tmem;
+  U.bars = bars;
+  U.c0 = U.c1 = U.c2 = U.c3 = U.g0 = U.g1 = 0;
+  U.abort = abort;
+  U.failed = false;
+  if constexpr (SPIN2)
+    u2_unit<NDER, MODE, NC, NB, NH>(D, m, rblk, sm, U);
+  else
+    u0_unit<NDER, MODE, NC, NB, NH>(D, m, rblk, sm, U);
+  return make_uint4(U.failed ? 1u : 0u, U.g0, U.g1, 0u);
+}
+
 // Persistent form: one launch covers the Legendre work of several plans. Items
 // (descriptor, kind, m, ring block) are pre-sorted by cost; each CTA takes them in
 // order from an atomic counter until none is left (no waits between CTAs). Kinds:
@@ -880,6 +900,9 @@ __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MO
   __shared__ uint32_t tbase;
   __shared__ int abort_flag;
   __shared__ int cur;
+  // the item's descriptor (a copy per thread would live in local memory)
+  __shared__ __align__(16) unsigned char dbuf[sizeof(TcDesc)];
+  const TcDesc &D = *(const TcDesc *)dbuf;
   typedef Tc<NDER, MODE> C;
   constexpr int NC = C::NC, NH = C::NH;
   typedef typename C::TM TM;
@@ -887,7 +910,13 @@ __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MO
   static_assert(TM1::A0 + NH * TM::NB * TM1::ASET <= TM::cols, "potential units fit the allocation");
   UmmaCta U;
   umma_open<TM::cols, TM::NB, NH>(U, bars, &tbase, &abort_flag);
-  TcDesc D = descs[0];
+  static_assert(sizeof(TcDesc) % 4 == 0, "copied in words");
+  auto take = [&](int d) {
+    for (int i = threadIdx.x; i < (int)(sizeof(TcDesc) / 4); i += blockDim.x)
+      ((int *)dbuf)[i] = __ldg((const int *)(descs + d) + i);
+    __syncthreads();
+  };
+  take(0);  // (umma_close reads it even if there is no item)
   for (;;) {
     __syncthreads();  // the previous item's readers of `cur` are done
     if (threadIdx.x == 0) cur = atomicAdd(counter, 1);
@@ -895,14 +924,25 @@ __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MO
     const int it = cur;
     if (it >= nitems) break;
     const int4 w = items[it];
-    D = descs[w.x & 0xffff];
+    // Every item starts on fresh barriers (all of the one before are idle: every MMA, copy and
+    // arrival has been waited for), so that its block counts start at 0 at compile time
+    if (threadIdx.x < 12 * NH) {
+      const uint32_t bar = smem_u32(&bars[threadIdx.x]), i = threadIdx.x % 12;
+      asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar),
+                   "r"((i == 2 || i == 3) ? 4 * NH / tc_groups(NH, TM::NB) : 1)
+                   : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    take(w.x & 0xffff);
     const int kind = w.x >> 16;
-    if (kind == 2)
-      u2_unit<NDER, MODE, NC, TM::NB, NH>(D, w.y, w.z, sm, U);
-    else if (kind == 1)
-      u0_unit<1, MODE, NC, TM::NB, NH>(D, w.y, w.z, sm, U);
-    else
-      u0_unit<NDER, MODE, NC, TM::NB, NH>(D, w.y, w.z, sm, U);
+    const uint4 q = kind == 2   ? unit_call<NDER, MODE, NC, TM::NB, NH, true>(&D, w.y, w.z, sm, U.tmem, U.bars, U.abort)
+                    : kind == 1 ? unit_call<1, MODE, NC, TM::NB, NH, false>(&D, w.y, w.z, sm, U.tmem, U.bars, U.abort)
+                                : unit_call<NDER, MODE, NC, TM::NB, NH, false>(&D, w.y, w.z, sm, U.tmem, U.bars, U.abort);
+    U.failed = q.x != 0;
+    U.g0 = q.y;
+    U.g1 = q.z;
     if (U.failed) break;  // uniform: set after a block-wide vote
   }
   umma_close<TM::cols, TM::NB, NH>(D, U);
