@@ -26,8 +26,8 @@
 // function of m modulo the length).
 //
 // What bounds it: instruction issue (the belt kernel 69%, the cap kernels 60-65% issue-active at 24-32
-// warps per SM, DRAM under 35% of its peak). Sixteen T+Q/U realisations of order 4 take 108 ms at
-// Nside 2048 / lmax 3000 and 10.8 ms at Nside 512 / lmax 1024, against 232 and 21.9 ms for packed
+// warps per SM, DRAM under 35% of its peak). Sixteen T+Q/U realisations of order 4 take 107 ms at
+// Nside 2048 / lmax 3000 and 10.0 ms at Nside 512 / lmax 1024, against 232 and 21.9 ms for packed
 // pairs of maps with Bluestein's convolution in the caps. Of this, one weight for a pixel and
 // its mirror image gave 6 ms at Nside 2048 (the cap kernels' instructions per map and pixel fell by
 // a fifth), and the packed twiddle table 19 ms (a warp's twiddle loads touched up to 88 lines
