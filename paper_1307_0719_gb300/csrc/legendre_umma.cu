@@ -483,7 +483,8 @@ template <int NC, int NH> __host__ __device__ constexpr uint32_t xch_offset() {
 // at Nside 2048 / lmax 3000 it takes 820 in the loop (the issuing warp shares its scheduler with
 // compute warps that are 67% issue-active, and waits 240 cycles per two blocks) and 950 with the unit's
 // start, end and epilogue. Before (two parts, the tiles through the compute warps' registers, one
-// lane per block): 1330. Spin 2 103.9 -> 74.3 ms, spin 0 with the potential 70.0 -> 52.6 ms.
+// lane per block): 1330. Spin 2 103.9 -> 73.0 ms, spin 0 with the potential 70.0 -> 51.5 ms (of which one
+// millisecond each from not storing the coefficients that every ring of a warp holds at zero).
 template <int NDER, int MODE, int NC, int NB, bool SPIN2, int NH>
 __device__ __forceinline__ int run_blocks(const TcDesc &D, int m, int rblk, unsigned char *sm, UmmaCta &U) {
   constexpr int NJ = NDER + 1;
@@ -969,8 +970,16 @@ __global__ void __launch_bounds__(kComputeThreads) tcstart_kernel(TcDesc D, int 
   const long long unit = (long long)m * D.nrblk + rblk;
   bool active;
   const int r = unit_ring<SPIN2>(D, rblk, tid, active);
+  // beyond mcut no ring ever leaves the gated range and no coefficient is stored
+  if (D.mcut && !__syncthreads_or(active && m <= D.mcut[r])) {
+    if (tid == 0) bstart[unit] = nblk;
+    return;
+  }
   Leib<float, NDER> LC;
-  leibniz_coefs<float, NDER>(D.rt.z[r], D.rt.sint[r], 1.0 / (double)(D.lmax + 1), LC);
+#pragma unroll
+  for (int j = 1; j <= NDER; ++j)
+#pragma unroll
+    for (int i = 1; i <= j; ++i) LC.e[j][i] = __ldg(D.leib + (size_t)(j * (j - 1) / 2 + i - 1) * D.nrings + r);
   float a[NJ], b[NJ];
   int sc;
   unit_seed<NDER, SPIN2>(D, r, m, active, a, b, sc);
