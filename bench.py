@@ -63,10 +63,10 @@ def fp32_peak_tflops(dev, peaks):
 # count (rings x m grows the same way); a changed source, another order or form
 # gives null.
 TRAFFIC_NSIDE512 = {
-    ("fft_total", None): (858.2e6, ['ringfft.cu', 'fft.cuh', 'regfft.cuh', 'common.cuh'], "331f595a91f2531e"),
+    ("fft_total", None): (638.9e6, ['ringsynth.cu', 'ringjobs.cuh', 'regfft.cuh', 'tables.cu', 'common.cuh'], "978d7348455c6ed1"),
     ("gather_total", None): (627.4e6, ['gather.cu', 'geometry.cuh'], "bcdaeea7440cc516"),
-    ("legendre_QU", "bf16x3"): (3.1023e9, ['legendre_umma.cu', 'legendre.cuh', 'common.cuh'], "1b171c4fa0306540"),
-    ("legendre_T", "bf16x3"): (2.4593e9, ['legendre_umma.cu', 'legendre.cuh', 'common.cuh'], "1b171c4fa0306540"),
+    ("legendre_QU", "bf16x3"): (2.4967e9, ['legendre_umma.cu', 'legendre.cuh', 'common.cuh'], "e919b44aa6f9d309"),
+    ("legendre_T", "bf16x3"): (2.0040e9, ['legendre_umma.cu', 'legendre.cuh', 'common.cuh'], "e919b44aa6f9d309"),
 }
 
 
@@ -322,7 +322,7 @@ def run_ours(args):
             continue  # a temperature-only workload has no spin-2 stage
         fl = legendre_flops_per_launch(w.nside, w.lmax, w.order, spin, part=part) * launches
         ach = fl / (stage_ms[st] / 1e3) / 1e12
-        e = {"kernel": f"legendre_spin{spin}_{'umma' if tc else 'kernel'}<{w.order}>", "bound": "alu",
+        e = {"kernel": f"legendre_spin{spin}_{'umma' if tc else 'f32_kernel'}<{w.order}>", "bound": "alu",
              "achieved": ach, "peak": fp32_peak, "unit": "TFLOP/s", "frac": ach / fp32_peak,
              "traffic": captured_traffic(st, w, 1, args.form) if (tc and nb == 16) else None,
              "peak_source": fp32_src,
@@ -337,7 +337,7 @@ def run_ours(args):
     npix = 12 * w.nside * w.nside
     fft_bytes = nchunk * (nplanes * nrings * (w.lmax + 1) * 8 + nmaps * npix * 4)
     gat_bytes = nchunk * npix * (nf * (w.order + 1) * (w.order + 2) // 2 * 4 + 2 * 4 + nf * 4)
-    for st, byt, kname in (("fft_total", fft_bytes, "ringfft_kernel<float> (all ring groups)"),
+    for st, byt, kname in (("fft_total", fft_bytes, "ringfft_synth_kernel (all ring groups)"),
                            ("gather_total", gat_bytes, f"gather_kernel<float, {w.order}, 1>")):
         ach = byt / (stage_ms[st] / 1e3) / 1e9 if stage_ms.get(st) else None
         rl[st] = {"kernel": kname, "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",
@@ -598,7 +598,7 @@ def run_adjoint(args, standalone=True):
         spin = 2 if dom == "legendre_QU_adj" else 0
         fl = legendre_flops_per_launch(w.nside, w.lmax, w.order, spin)
         ach = fl / (stage_ms[dom] / 1e3) / 1e12
-        roof = {"kernel": f"legendre_adj{spin}_kernel<float, {w.order}>", "bound": "alu", "achieved": ach,
+        roof = {"kernel": f"legendre_adj{spin}_f32_kernel<{w.order}>", "bound": "alu", "achieved": ach,
                 "peak": fp32_peak, "unit": "TFLOP/s", "frac": ach / fp32_peak, "traffic": None,
                 "peak_source": fp32_src,
                 "counts": "recurrence + transposed contraction (same per-triple count as the forward)"}
@@ -625,6 +625,9 @@ def run_adjoint(args, standalone=True):
     gr = step(d)
     torch.cuda.synchronize()
     gnorm = {k: float(v.abs().pow(2).sum().sqrt()) for k, v in gr.items()}
+    # forward call; then the adjoint's recomputed maps (a forward call without its two gather
+    # launches), transposed gather, ten ring-FFT groups, two Legendre launches, finish
+    launches_per_step = 2 * plan.batch_launches(1) + 12
     plan.close()
     cpu = None
     if rank == 0 and not args.no_cpu_baseline:
@@ -655,7 +658,7 @@ def run_adjoint(args, standalone=True):
                        "parallelism": f"replicas{world}",
                        "l2": "inputs larger than L2 (derivative maps 2.3 GB, their gradients 2.3 GB)"},
             "stage_ms": stage_ms, "roofline": roof, "clocks": clk.summary(),
-            "gpu_launches": args.steps * 20, "e2e": e2e, "grad_norms": gnorm, "cpu_baseline": cpu,
+            "gpu_launches": args.steps * launches_per_step, "e2e": e2e, "grad_norms": gnorm, "cpu_baseline": cpu,
         }
     if world > 1 and standalone:
         dist.destroy_process_group()
