@@ -646,13 +646,17 @@ __device__ __forceinline__ int run_blocks(const TcDesc &D, int m, int rblk, unsi
   if (NH > 2) U.c3 += (uint32_t)count_of(3);
   U.g0 += (uint32_t)handoffs(0);
   if (NG > 1) U.g1 += (uint32_t)handoffs(NG - 1);
-  // the last commit of each group covers every MMA issued before it
+  // the last commit of each group covers every MMA issued before it; with two buffers the other buffer's
+  // barrier gets the arrival of the commit before, which has to be in too before the barriers are
+  // initialised anew (legendre_umma_persistent)
 #pragma unroll
   for (int gr = 0; gr < NG; ++gr) {
     const uint32_t c = group_count(U, gr);
-    if (!bad && handoffs(gr) > 0 &&
-        !mbar_wait(bar_done(U, buf_of<NB>(c - 1), gr), phase_of<NB>(c - 1), D.polls, U.abort))
-      bad = true;
+#pragma unroll
+    for (int b = 1; b <= NB; ++b)
+      if (!bad && handoffs(gr) >= b &&
+          !mbar_wait(bar_done(U, buf_of<NB>(c - b), gr), phase_of<NB>(c - b), D.polls, U.abort))
+        bad = true;
   }
   // the parts' last stages are free too (every block frees its stage once)
 #pragma unroll
