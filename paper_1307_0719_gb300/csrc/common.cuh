@@ -59,10 +59,11 @@ struct SyGroup {
   int mode, lg, first, count, band;
 };
 #define TL_MAX_SY_GROUPS 16
-constexpr int kSyCorr = 5120;  // entries of each window's correction table
+constexpr int kSyCorr = 4097;  // entries of the window's correction table: up to a quarter of a grid of 2^14
+constexpr int kSyW = 10;       // taps of the interpolation window
 // interpolation window: per tap of the first half, the polynomial's coefficients in s
 struct SyWindow {
-  float c10[5][9], c8[4][9];
+  float c[kSyW / 2][9];
 };
 
 }  // namespace tl
@@ -94,7 +95,7 @@ struct tl_plan {
   tl::SyGroup sy_groups[TL_MAX_SY_GROUPS];
   int4 *sy_rings;       // {ring, band, fold, mcut} by group (device)
   float4 *sy_tw4;       // twiddles of the synthesis transforms (host_synth_twiddles)
-  float *sy_corr;       // [2][kSyCorr] corrections of the two windows (device)
+  float *sy_corr;       // [kSyCorr] corrections of the window (device)
   tl::SyWindow sy_win;
   int *rest_rings;      // ring indices of rest_groups (device)
   tl::FftGroup rest_groups[TL_MAX_FFT_GROUPS];
@@ -271,12 +272,12 @@ int host_fft_groups(int nside, int nrings, const int *nphi, const int *ml, FftGr
 // below 2^-h being held at zero
 void host_ring_bands(int nside, int lmax, int h, const double *sint, const double *z, int *mcut);
 struct JobList;
-// entries (eight floats each) of the synthesis kernels' twiddle table, filled when out is given
+// entries (four floats each) of the synthesis kernels' twiddle table, filled when out is given
 int host_synth_twiddles(float *out);
-const float *host_synth_window(SyWindow *w);  // returns [2][kSyCorr] corrections
+const float *host_synth_window(SyWindow *w);  // returns [kSyCorr] corrections
 int host_synth_groups(int nside, int nrings, const int *nphi, const int *mcut, SyGroup *groups, int4 *rings, int *rest,
                       int *nrest);
-cudaError_t launch_ring_synth(const tl_plan *p, const JobList &jl, cudaStream_t s);
+cudaError_t launch_ring_synth(const tl_plan *p, JobList &jl, cudaStream_t s);  // (sets the jobs' scalef)
 cudaError_t raise_smem(const void *fn, size_t bytes);
 cudaError_t launch_bluestein_setup_impl(tl_plan *p, const double2 *tw64, cudaStream_t s);
 

@@ -181,10 +181,10 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
       TRY_CUDA(upload(&p->rest_rings, order, B));
     }
     const float *cw = host_synth_window(&p->sy_win);
-    std::vector<float> corr(cw, cw + 2 * (size_t)kSyCorr);
+    std::vector<float> corr(cw, cw + kSyCorr);
     TRY_CUDA(upload(&p->sy_rings, rings, B));
     TRY_CUDA(upload(&p->sy_corr, corr, B));
-    std::vector<float> tw4(8 * (size_t)host_synth_twiddles(nullptr));
+    std::vector<float> tw4(4 * (size_t)host_synth_twiddles(nullptr));
     host_synth_twiddles(tw4.data());
     TRY_CUDA(upload((float **)&p->sy_tw4, tw4, B));
     for (int i = 0; i < p->sy_ngroups; ++i) sy_tw = sy_tw > (4 << p->sy_groups[i].lg) ? sy_tw : (4 << p->sy_groups[i].lg);

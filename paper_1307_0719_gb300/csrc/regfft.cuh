@@ -122,38 +122,75 @@ __device__ __forceinline__ void dft_small(float2 *a) {
 __device__ __forceinline__ int rpad(int a) { return a + (a >> 4); }
 __device__ __forceinline__ float2 conj_if(float2 a, bool c) { return c ? f2(a.x, -a.y) : a; }
 
-// Where a pass takes W_L^j, W_L^2j, W_L^4j and W_L^8j (j < L / 16, sign DIR) from:
-// the plan's table tw[k] = e^{-2 pi i k / TW}, k < TW / 2
+// y_q *= W_L^{j q}, q = 1..15, from four values (j, 2j, 4j, 8j) and products of at most three of them
+__device__ __forceinline__ void twiddle16(float2 (&x)[16], float2 w1, float2 w2, float2 w4, float2 w8) {
+  const float2 w3 = cmul(w1, w2), w5 = cmul(w1, w4), w6 = cmul(w2, w4), w7 = cmul(w3, w4);
+  x[1] = cmul(x[1], w1);
+  x[2] = cmul(x[2], w2);
+  x[3] = cmul(x[3], w3);
+  x[4] = cmul(x[4], w4);
+  x[5] = cmul(x[5], w5);
+  x[6] = cmul(x[6], w6);
+  x[7] = cmul(x[7], w7);
+  x[8] = cmul(x[8], w8);
+  x[9] = cmul(x[9], cmul(w1, w8));
+  x[10] = cmul(x[10], cmul(w2, w8));
+  x[11] = cmul(x[11], cmul(w3, w8));
+  x[12] = cmul(x[12], cmul(w4, w8));
+  x[13] = cmul(x[13], cmul(w5, w8));
+  x[14] = cmul(x[14], cmul(w6, w8));
+  x[15] = cmul(x[15], cmul(w7, w8));
+}
+
+// Where a pass takes its twiddles W_L^{j q} (j < L / 16, q = 1..15, sign DIR) from:
+// the plan's table tw[k] = e^{-2 pi i k / TW}, k < TW / 2, four of them, and products of these
 template <int DIR> struct TwidTable {
   const float2 *__restrict__ tw;
   int lgtw;
   template <int LG, int P>
-  __device__ __forceinline__ void get(int j, float2 &w1, float2 &w2, float2 &w4, float2 &w8) const {
+  __device__ __forceinline__ void apply(float2 (&x)[16], int j) const {
     const int s = j << (lgtw - (LG - 4 * P));
     const bool cj = DIR > 0;
-    w1 = conj_if(__ldg(tw + s), cj);
-    w2 = conj_if(__ldg(tw + 2 * s), cj);
-    w4 = conj_if(__ldg(tw + 4 * s), cj);
-    w8 = conj_if(__ldg(tw + 8 * s), cj);
+    twiddle16(x, conj_if(__ldg(tw + s), cj), conj_if(__ldg(tw + 2 * s), cj), conj_if(__ldg(tw + 4 * s), cj),
+              conj_if(__ldg(tw + 8 * s), cj));
   }
 };
-// or a table of the four side by side per pass (DIR = +1), pass by pass: 32 bytes per j, so that a
-// warp's loads touch 8 lines a pass (their scattered entries of tw lie in up to 88)
+// or a table of six (q = 1, 2, 3, 4, 8, 12; DIR = +1), pass by pass, so that every other one is a single
+// product: a float transform's error falls by a seventh against four and products of up to three (1.40e-7 ->
+// 1.28e-7 relative RMS on the belt rings at Nside 512 to 2048) at the same time. Three rows of L / 16 pairs, so that
+// a warp's loads are contiguous (the scattered entries of tw lie in up to 88 lines; all fifteen from a table
+// took 6% more of the whole synthesis at Nside 2048).
 struct TwidPacked {
+  static constexpr int PER = 3;  // float4 per j
   const float4 *__restrict__ t;
-  // entries of the passes before pass P
+  // values of j of the passes before pass P
   template <int LG> __host__ __device__ static constexpr int offset(int P) {
     int n = 0;
     for (int i = 0; i < P; ++i) n += 1 << (LG - 4 * i - 4);
     return n;
   }
   template <int LG, int P>
-  __device__ __forceinline__ void get(int j, float2 &w1, float2 &w2, float2 &w4, float2 &w8) const {
-    const float4 a = __ldg(t + 2 * (offset<LG>(P) + j)), b = __ldg(t + 2 * (offset<LG>(P) + j) + 1);
-    w1 = f2(a.x, a.y);
-    w2 = f2(a.z, a.w);
-    w4 = f2(b.x, b.y);
-    w8 = f2(b.z, b.w);
+  __device__ __forceinline__ void apply(float2 (&x)[16], int j) const {
+    constexpr int NJ = 1 << (LG - 4 * P - 4);
+    const float4 *tp = t + PER * offset<LG>(P) + j;
+    const float4 a = __ldg(tp), b = __ldg(tp + NJ), c = __ldg(tp + 2 * NJ);
+    const float2 w1 = f2(a.x, a.y), w2 = f2(a.z, a.w), w3 = f2(b.x, b.y), w4 = f2(b.z, b.w), w8 = f2(c.x, c.y),
+                 w12 = f2(c.z, c.w);
+    x[1] = cmul(x[1], w1);
+    x[2] = cmul(x[2], w2);
+    x[3] = cmul(x[3], w3);
+    x[4] = cmul(x[4], w4);
+    x[5] = cmul(x[5], cmul(w4, w1));
+    x[6] = cmul(x[6], cmul(w4, w2));
+    x[7] = cmul(x[7], cmul(w4, w3));
+    x[8] = cmul(x[8], w8);
+    x[9] = cmul(x[9], cmul(w8, w1));
+    x[10] = cmul(x[10], cmul(w8, w2));
+    x[11] = cmul(x[11], cmul(w8, w3));
+    x[12] = cmul(x[12], w12);
+    x[13] = cmul(x[13], cmul(w12, w1));
+    x[14] = cmul(x[14], cmul(w12, w2));
+    x[15] = cmul(x[15], cmul(w12, w3));
   }
 };
 
@@ -165,29 +202,6 @@ struct RegFft {
   static constexpr int NPASS = NP16 + (RL > 1 ? 1 : 0);
   static constexpr int SMEM = N + (N >> 4);        // padded elements of the exchange array
   static_assert(LG >= 8, "at least two radix-16 passes");
-
-  // y_q *= W_L^{j q}, q = 1..15: four table values (j, 2j, 4j, 8j) and products of at most three
-  // of them
-  template <int P, typename TW> __device__ static void twiddle(float2 (&x)[16], int j, TW tw) {
-    float2 w1, w2, w4, w8;
-    tw.template get<LG, P>(j, w1, w2, w4, w8);
-    const float2 w3 = cmul(w1, w2), w5 = cmul(w1, w4), w6 = cmul(w2, w4), w7 = cmul(w3, w4);
-    x[1] = cmul(x[1], w1);
-    x[2] = cmul(x[2], w2);
-    x[3] = cmul(x[3], w3);
-    x[4] = cmul(x[4], w4);
-    x[5] = cmul(x[5], w5);
-    x[6] = cmul(x[6], w6);
-    x[7] = cmul(x[7], w7);
-    x[8] = cmul(x[8], w8);
-    x[9] = cmul(x[9], cmul(w1, w8));
-    x[10] = cmul(x[10], cmul(w2, w8));
-    x[11] = cmul(x[11], cmul(w3, w8));
-    x[12] = cmul(x[12], cmul(w4, w8));
-    x[13] = cmul(x[13], cmul(w5, w8));
-    x[14] = cmul(x[14], cmul(w6, w8));
-    x[15] = cmul(x[15], cmul(w7, w8));
-  }
 
   template <int P, typename TW> __device__ static void pass(float2 (&x)[16], float2 *sm, int h, TW tw) {
     constexpr bool R16 = P < NP16;
@@ -226,7 +240,7 @@ struct RegFft {
     if constexpr (!LAST) {
       static_assert(G == 1, "only the last pass may be shorter");
       const int j = h & (m - 1), Q = h >> lgm;
-      twiddle<P>(x, j, tw);
+      tw.template apply<LG, P>(x, j);
       if constexpr (P == 0) __syncthreads();  // the array's previous readers are done
       const int pb = rpad(Q * m + j);
       constexpr int st = S * m + ((S * m) >> 4);  // S m is a multiple of 16

@@ -10,27 +10,31 @@
 //
 // Rings whose pixels are grid points (the belt: 4 Nside a power of two) store z_n at
 // once. The cap rings have 4 i pixels; their function of longitude is band limited (m <= band),
-// so it is sampled on an oversampled power-of-two grid and interpolated to the pixels with a
-// Kaiser-Bessel window of W grid points, the coefficients having been divided by the
-// window's transform (gridding; Jackson et al. 1991, IEEE Trans. Med. Imaging 10, 473). W = 10 at an
-// oversampling of at least 1.65 and W = 8 at 2 or more leave a relative error of 1e-8 and
-// 4e-8, below the rounding of the transform itself. This takes one transform of about
-// the ring's own length per map; Bluestein's chirp-z convolution, exact for any length, takes
-// four of 2 to 4 times the sub-sequence length each (per map of a packed pair).
+// so it is sampled on a power-of-two grid that oversamples it at least twice and interpolated to the pixels
+// with a Kaiser-Bessel window of W = 10 grid points, the coefficients having been divided by the
+// window's transform (gridding; Jackson et al. 1991, IEEE Trans. Med. Imaging 10, 473). The method's own
+// error is 3e-9 at the band's edge; what counts is the transform's float rounding, which the division
+// amplifies at the top of the band (by 3.7 at an oversampling of 2, by 8 at 1.65). Relative RMS error of a map,
+// of the rings' rows alone (coefficients ~ (m + 1)^p, p = -1 .. 2, phi-derivatives 0 .. 4, Nside 64 to 2048): caps 1.07 to
+// 1.68e-7, no map of a ring above 2.2e-7, belt 1.18 to 1.37e-7. Packed pairs of maps with Bluestein's convolution in
+// the caps: 1.41 to 2.5e-7, belt 1.05 to 1.7e-7, and up to 9e-6 where a map shared its transform with a much larger
+// one. An oversampling of 1.65 with W = 8 for `twice`: 1.9 to 4.3e-7 on the rings next below a larger
+// grid, for 9% less time at Nside 2048; 1.9 instead of 2 up to 12% above Bluestein on single rings, for 3%.
+// This takes one transform of one to two times the ring's own length per map; Bluestein's chirp-z
+// convolution, exact for any length, takes four of 2 to 4 times the sub-sequence length each (per map of a packed pair).
 //
 // The rows of F are zero beyond the ring's mcut (see host_ring_bands): the Legendre stage holds
 // functions below 2^-32 at zero. Nothing beyond is read. Rows are staged
 // once per plane in shared memory, scaled by the window's correction, and multiplied by
-// i m / L from one phi-derivative to the next. Where the band limit exceeds half the
+// i m / P (a power of two, see synth_power) from one phi-derivative to the next. Where the band limit exceeds half the
 // ring's length the aliases are folded while staging (per map, since (m / L)^k is not a
 // function of m modulo the length).
 //
-// What bounds it: instruction issue (the belt kernel 69%, the cap kernels 60-65% issue-active at 24-32
-// warps per SM, DRAM under 35% of its peak). Sixteen T+Q/U realisations of order 4 take 107 ms at
-// Nside 2048 / lmax 3000 and 10.0 ms at Nside 512 / lmax 1024, against 232 and 21.9 ms for packed
-// pairs of maps with Bluestein's convolution in the caps. Of this, one weight for a pixel and
-// its mirror image gave 6 ms at Nside 2048 (the cap kernels' instructions per map and pixel fell by
-// a fifth), and the packed twiddle table 19 ms (a warp's twiddle loads touched up to 88 lines
+// What bounds it: instruction issue. Sixteen T+Q/U realisations of order 4 take 118 ms at
+// Nside 2048 / lmax 3000 and 10.4 ms at Nside 512 / lmax 1024, against 232 and 21.9 ms for packed
+// pairs of maps with Bluestein's convolution in the caps. One weight for a pixel and
+// its mirror image took 6 ms off at Nside 2048 (the cap kernels' instructions per map and pixel fell by
+// a fifth), and packed twiddle tables 19 ms (a warp's twiddle loads touched up to 88 lines
 // a pass, as much of the load path's time as all shared-memory traffic).
 #include <math.h>
 
@@ -59,10 +63,9 @@ __device__ __constant__ float2 kRoot64[32] = {
 
 // Modes of a ring group:
 //  direct  the ring's pixels are every (2H / N)-th grid point (N = 4 Nside <= 2H);
-//  single  one grid of 2H points, oversampled at least 1.65 times, W = 10;
+//  single  one grid of 2H points, at least twice the band's own;
 //  twice   the largest rings: two grids of 2H points half a step apart (two transforms of
-//          length H = 4096 by two groups of threads), together a grid of 4H points
-//          oversampled at least twice, W = 8.
+//          length H = 4096 by two groups of threads), together a grid of 4H points.
 enum { kSyDirect = 0, kSySingle = 1, kSyTwice = 2 };
 
 // TG = H / 16 threads hold one transform; a CTA of NT threads holds G of them on one
@@ -75,7 +78,7 @@ template <int LG, int MODE> struct SyCfg {
   static constexpr int CTAS = MODE == kSyDirect ? (LG == 12 ? 3 : 4) : (LG >= 11 ? 2 : LG == 8 ? 8 : 4);
   static constexpr int G = NT / TG;
   static constexpr int MAPS = MODE == kSyTwice ? 1 : G;  // maps of a CTA at a time
-  static constexpr int W = MODE == kSyTwice ? 8 : 10;
+  static constexpr int W = kSyW;
   static constexpr int X = RegFft<LG, +1>::SMEM;  // float2 of an exchange array
 };
 
@@ -176,7 +179,7 @@ __global__ void __launch_bounds__(SyCfg<LG, MODE>::NT, SyCfg<LG, MODE>::CTAS)
       if (J.in == pin && k == pk + 1 && !fold) {
         for (int m = sm0; m <= band; m += sms) {
           const float2 v = row[m];
-          const float mm = (float)m * A.invL;
+          const float mm = (float)m * A.invL;  // exact
           row[m] = f2(-v.y * mm, v.x * mm);
         }
       } else {
@@ -331,8 +334,8 @@ __global__ void __launch_bounds__(SyCfg<LG, MODE>::NT, SyCfg<LG, MODE>::CTAS)
         float wt[W];
 #pragma unroll
         for (int t = 0; t < HW; ++t) {
-          const float *pc = W == 10 ? win.c10[t] : win.c8[t];
-          constexpr int NE = W == 10 ? 5 : 4, NO = 4;  // even and odd coefficients
+          const float *pc = win.c[t];
+          constexpr int NE = 5, NO = 4;  // even and odd coefficients
           float e = pc[2 * (NE - 1)], o = pc[2 * NO - 1];
 #pragma unroll
           for (int i = NE - 2; i >= 0; --i) e = fmaf(e, s2, pc[2 * i]);
@@ -444,23 +447,18 @@ static void kb_poly(int W, double beta, double c0, int D, float *out) {
   for (int i = 0; i < n; ++i, s *= 2.0) out[i] = (float)(p[i] * s);
 }
 
-constexpr double kSigma10 = 1.65, kSigma8 = 2.0;
+constexpr double kSigma = 2.0;  // oversampling of a band at least
 
-// Window polynomials, and the correction tables: corr[m] of W = 10 at m / 2^14 for m <= 2^13 /
-// kSigma10, then of W = 8 for m <= 2^13 / kSigma8 (kSyCorr entries each). They depend on nothing:
+// Window polynomials, and the correction corr[m] at m / 2^14 of a grid (a band is at most the
+// (2 kSigma)-th part of its grid: kSyCorr entries). They depend on nothing:
 // formed once per process.
 struct SynthWindow {
   SyWindow win;
-  float corr[2 * kSyCorr];
+  float corr[kSyCorr];
   SynthWindow() {
-    const double b10 = kb_beta(10, kSigma10), b8 = kb_beta(8, kSigma8);
-    for (int t = 0; t < 5; ++t) kb_poly(10, b10, t - 4.5, 8, win.c10[t]);
-    for (int t = 0; t < 4; ++t) kb_poly(8, b8, t - 3.5, 7, win.c8[t]);
-    for (int t = 0; t < 4; ++t) win.c8[t][8] = 0.0f;
-    for (int m = 0; m < kSyCorr; ++m) {
-      corr[m] = (float)(1.0 / kb_transform(m / 16384.0, 10, b10));
-      corr[kSyCorr + m] = (float)(1.0 / kb_transform(m / 16384.0, 8, b8));
-    }
+    const double beta = kb_beta(kSyW, kSigma);
+    for (int t = 0; t < kSyW / 2; ++t) kb_poly(kSyW, beta, t - 0.5 * (kSyW - 1), 8, win.c[t]);
+    for (int m = 0; m < kSyCorr; ++m) corr[m] = (float)(1.0 / kb_transform(m / 16384.0, kSyW, beta));
   }
 };
 const float *host_synth_window(SyWindow *w) {
@@ -478,24 +476,29 @@ static constexpr int synth_twiddle_offset(int lg) {
 }
 int host_synth_twiddles(float *out) {
   const int n = synth_twiddle_offset(13);
-  if (!out) return n;
+  if (!out) return n * TwidPacked::PER;
   for (int g = 8; g <= 12; ++g) {
-    float *o = out + 8 * (size_t)synth_twiddle_offset(g);
+    float *o = out + 4 * TwidPacked::PER * (size_t)synth_twiddle_offset(g);
     for (int p = 0; 4 * p + 4 <= g; ++p) {
       const int L = 1 << (g - 4 * p);
-      for (int j = 0; j < L / 16; ++j, o += 8)
-        for (int q = 0; q < 4; ++q) {
-          const double a = 2.0 * M_PI * (double)(j << q) / (double)L;
-          o[2 * q] = (float)cos(a);
-          o[2 * q + 1] = (float)sin(a);
+      const int nj = L / 16;
+      for (int j = 0; j < nj; ++j) {
+        const int qs[6] = {1, 2, 3, 4, 8, 12};
+        for (int q = 0; q < 6; ++q) {
+          const double a = 2.0 * M_PI * (double)(j * qs[q]) / (double)L;
+          float *w = o + 4 * (size_t)((q / 2) * nj + j) + 2 * (q & 1);
+          w[0] = (float)cos(a);
+          w[1] = (float)sin(a);
         }
+      }
+      o += 12 * (size_t)nj;
     }
   }
   return n;
 }
 
 // Group of one ring, by its length and band (mcut: its coefficients beyond are zero):
-// the belt on its own grid; the caps on the smallest grid that oversamples their band,
+// the belt on its own grid; the caps on the smallest grid that oversamples their band kSigma times,
 // which is half the ring's length where folding the aliases buys a smaller grid.
 // Returns the group key (mode and log2 H), -1 if no grid fits; sets band and fold.
 static int synth_key(int nside, int nphi, int mcut, int *band, int *fold) {
@@ -513,7 +516,7 @@ static int synth_key(int nside, int nphi, int mcut, int *band, int *fold) {
   }
   auto grid = [](int b) {
     for (int lg = 8; lg <= 12; ++lg)
-      if ((double)(2 << lg) >= kSigma10 * 2.0 * b) return kSySingle * 16 + lg;
+      if ((double)(2 << lg) >= kSigma * 2.0 * b) return kSySingle * 16 + lg;
     return b <= 4095 ? kSyTwice * 16 + 12 : -1;
   };
   int key = grid(mcut);
@@ -557,6 +560,15 @@ int host_synth_groups(int nside, int nrings, const int *nphi, const int *mcut, S
 
 // ---------------------------------------------------------------------------
 
+// The kernels' phi-derivative factor is m / P for the power of two P >= lmax + 1: exact in float, so that
+// the k-th derivative's coefficients round k times instead of carrying the k-fold rounding of m / L (and of
+// 1 / L, the same for all m). (P / L)^k goes into the map's scale.
+static double synth_power(int lmax) {
+  double P = 1.0;
+  while (P < lmax + 1.0) P *= 2.0;
+  return P;
+}
+
 template <int LG, int MODE>
 static cudaError_t synth_launch(const tl_plan *p, const SyGroup &g, const JobList &jl, bool overlap,
                                 cudaStream_t s) {
@@ -568,12 +580,12 @@ static cudaError_t synth_launch(const tl_plan *p, const SyGroup &g, const JobLis
   A.rsinf = p->ring.rsinf;
   A.rings = p->sy_rings + g.first;
   A.tw = (const float2 *)p->twiddle;
-  A.tw4 = p->sy_tw4 + 2 * synth_twiddle_offset(LG);
-  A.corr = MODE == kSyTwice ? p->sy_corr + kSyCorr : p->sy_corr;
+  A.tw4 = p->sy_tw4 + TwidPacked::PER * synth_twiddle_offset(LG);
+  A.corr = p->sy_corr;
   A.lgtw = 31 - __builtin_clz((unsigned)p->tw_len);
   A.mmax = p->mmax;
   A.rowcap = (g.band + 2) & ~1;
-  A.invL = (float)(1.0 / (double)(p->lmax + 1));
+  A.invL = (float)(1.0 / synth_power(p->lmax));
   A.tile = 0;
   for (int i = 0; i < jl.n; ++i)
     if (jl.job[i].tile) {
@@ -614,7 +626,9 @@ static cudaError_t synth_launch(const tl_plan *p, const SyGroup &g, const JobLis
 // so every block waits for the group before at its end: the groups then complete in order. The
 // blocks that wait have all been placed, and those they wait for have all started. Up to Nside 1024: sixteen skies at Nside 512 take
 // 10.0 instead of 10.6 ms, but at Nside 2048, where the ends weigh little, 109.7 instead of 107.6.
-cudaError_t launch_ring_synth(const tl_plan *p, const JobList &jl, cudaStream_t s) {
+cudaError_t launch_ring_synth(const tl_plan *p, JobList &jl, cudaStream_t s) {
+  const double c = synth_power(p->lmax) / (double)(p->lmax + 1);
+  for (int i = 0; i < jl.n; ++i) jl.job[i].scalef = (float)(jl.job[i].scale * pow(c, jl.job[i].k));
   for (int i = 0; i < p->sy_ngroups; ++i) {
     const SyGroup &g = p->sy_groups[i];
     cudaError_t e = cudaErrorInvalidValue;
