@@ -155,7 +155,7 @@ extern "C" tl_status tl_batch_create(int nreal, const int *nside, const int *lma
     int g;
     if (it == gid.end()) {
       tl_plan *p = nullptr;
-      tl_status st = tl_plan_create(nside[i], lmax[i], order, spins, precision, flags, &p);
+      tl_status st = plan_create(nside[i], lmax[i], order, spins, precision, flags, 1, &p);
       if (st != TL_OK) {
         batch_free(b);
         return st;

@@ -114,7 +114,8 @@ struct tl_plan {
   // recurrence state there
   int *tc_bs0, *tc_bsp, *tc_bs2;
   float *tc_st0, *tc_stp, *tc_st2;
-  float *tc_sm0, *tc_smp, *tc_sm2;  // the same state at the first blocks of each unit's quarters 1 .. 3
+  float *tc_sm0, *tc_smp, *tc_sm2;  // the same state at the first blocks of each unit's later parts (tc_part_tables)
+  int tc_persistent;                // the plan's Legendre work runs in tl_batch's persistent launch too
   float *tc_leib;                   // Leibniz coefficients per ring
   float *tc_step0, *tc_step2;     // per 8-l block: A_{l+1} x 8, then A - 2 x 8 (spin 0) or Qn, Qs x 8 (spin 2)
   void *tc_b0, *tc_bp, *tc_b2;    // [blocks] 2 KB coefficient tiles (TF32 hi, lo; 32 columns x 8 l)
@@ -155,6 +156,10 @@ namespace tl {
 
 inline long long nalm(int lmax) { return (long long)(lmax + 1) * (lmax + 2) / 2; }
 inline int maps_per_field(int order) { return (order + 1) * (order + 2) / 2; }
+
+// tl_plan_create; persistent: with the tables of tl_batch's persistent Legendre launch
+tl_status plan_create(int nside, int lmax, int order, int spins, int precision, int flags, int persistent,
+                      tl_plan **out);
 
 // kernel launchers (defined in the .cu files)
 cudaError_t launch_steptab(const tl_plan *p, int s, void *tab, cudaStream_t st);
@@ -234,6 +239,7 @@ cudaError_t launch_legendre_spin0_tc(const tl_plan *p, int which, int nreal, voi
 // start tables of the tensor-core Legendre stage (which: 0 T, 1 potential, 2 Q/U)
 cudaError_t launch_tcstart(const tl_plan *p, int which, int *bstart, float *state, float *state_mid,
                            cudaStream_t s);
+int tc_part_tables(const tl_plan *p, int which);
 size_t tc_leib_bytes(const tl_plan *p);
 cudaError_t launch_tcleib(const tl_plan *p, float *out, cudaStream_t s);
 size_t tc_start_state_bytes(const tl_plan *p, int which);

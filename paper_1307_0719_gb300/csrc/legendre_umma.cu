@@ -265,10 +265,12 @@ struct TcDesc {
   // state at the start of that block: [unit][2 NJ + 1][128] (a, b, scale)
   const int *bstart;
   const float *state;
-  // the same state at the first block of the unit's quarters 1 .. 3 (seg_first), one
-  // array after another, mid_stride elements each; or NULL (no split)
+  // the same state at the first block of the unit's quarters 1 .. 3 (seg_first), or of its second
+  // half alone (mid_tables 3 or 1, see tc_part_tables), one array after another, mid_stride elements
+  // each; or NULL (no split)
   const float *state_mid;
   long long mid_stride;
+  int mid_tables;
   const float *leib;             // Leibniz coefficients e[j][i] per ring (leib_table_kernel)
   // [nrings] or NULL: coefficients of m > mcut[ring] (zeros) are not stored, because the ring
   // synthesis does not read them
@@ -596,8 +598,8 @@ __device__ __forceinline__ int run_blocks(const TcDesc &D, int m, int rblk, unsi
     int sc;
     if (D.bstart) {
       // the state at the part's first block, as the recurrence from l0 leaves it
-      const float *st = (h ? D.state_mid + (h * (4 / NH) - 1) * D.mid_stride : D.state) +
-                        unit * (2 * NJ + 1) * kComputeThreads + t;
+      const int q = NH == 4 ? h - 1 : D.mid_tables == 3 ? 1 : 0;
+      const float *st = (h ? D.state_mid + q * D.mid_stride : D.state) + unit * (2 * NJ + 1) * kComputeThreads + t;
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
         a[j] = __ldg(st + j * kComputeThreads);
@@ -956,8 +958,8 @@ __global__ void __launch_bounds__(umma_threads(Tc<NDER, MODE>::NH), (Tc<NDER, MO
 // Plan-time start table (see TcDesc): one CTA of 128 threads per unit runs the
 // recurrence block by block, without the contraction, until one of its rings has
 // reached scale 0 (a basis value that is not gated off), and records every ring's
-// state at the start of that block, bs. With state_mid it runs on and records the state at the
-// first block of the unit's quarters 1 .. 3 too. The launch kernels resume from these with the
+// state at the start of that block, bs. With `tables` part tables it runs on and records the state at the
+// first block of the unit's quarters 1 .. 3 (3) or of its second half (1) too. The launch kernels resume from these with the
 // same arithmetic (a warp holds the same 32 rings, so even the warp-uniform choices agree), so
 // their results are those of a run from l0. Units in which no ring contributes get
 // bstart = their block count.
@@ -965,7 +967,7 @@ template <int NDER, bool SPIN2>
 __global__ void __launch_bounds__(kComputeThreads) tcstart_kernel(TcDesc D, int *__restrict__ bstart,
                                                                    float *__restrict__ state,
                                                                    float *__restrict__ state_mid,
-                                                                   long long mid_stride) {
+                                                                   long long mid_stride, int tables) {
   constexpr int NJ = NDER + 1;
   const int rblk = blockIdx.x, m = blockIdx.y, tid = threadIdx.x;
   const int l0 = unit_l0(m, SPIN2);
@@ -1005,7 +1007,8 @@ __global__ void __launch_bounds__(kComputeThreads) tcstart_kernel(TcDesc D, int 
       // (a, b, sc) are the state at the start of this block
 #pragma unroll
       for (int q = 1; q < 4; ++q)
-        if (blk == first + seg_first(nblk - first, q)) record(state_mid + (q - 1) * mid_stride + so, a, b, sc);
+        if ((tables == 3 || q == 2) && blk == first + seg_first(nblk - first, q))
+          record(state_mid + (tables == 3 ? q - 1 : 0) * mid_stride + so, a, b, sc);
     }
     if (blk == stop) break;
     const float4 *stp = (const float4 *)(D.step + (b0 + blk) * step_stride(SPIN2));
@@ -1026,8 +1029,8 @@ __global__ void __launch_bounds__(kComputeThreads) tcstart_kernel(TcDesc D, int 
     if (first == nblk && __syncthreads_or(sc == 0)) {
       first = blk;
       record(state + so, sa, sb, ssc);
-      if (!state_mid) break;
-      stop = first + seg_first(nblk - first, 3);
+      if (!tables) break;
+      stop = first + seg_first(nblk - first, tables == 3 ? 3 : 2);
     }
   }
   if (tid == 0) bstart[unit] = first;
@@ -1236,6 +1239,7 @@ static TcDesc make_desc(const tl_plan *p, int which, int nreal, const void *btil
   D.mcut = p->sy_ngroups > 0 && p->rest_ngroups == 0 ? p->mcut : nullptr;
   D.leib = p->tc_leib;
   D.mid_stride = (long long)(tc_start_state_bytes(p, which) / sizeof(float));
+  D.mid_tables = tc_part_tables(p, which);
   D.bstart = which == 2 ? p->tc_bs2 : which == 1 ? p->tc_bsp : p->tc_bs0;
   D.state = which == 2 ? p->tc_st2 : which == 1 ? p->tc_stp : p->tc_st0;
   D.state_mid = which == 2 ? p->tc_sm2 : which == 1 ? p->tc_smp : p->tc_sm0;
@@ -1354,6 +1358,7 @@ cudaError_t launch_tcstart(const tl_plan *p, int which, int *bstart, float *stat
   D.state = nullptr;
   D.state_mid = nullptr;
   const long long ms = D.mid_stride;
+  const int tables = D.mid_tables;
   const int spin = which == 2 ? 2 : 0;
   const int nder = which == 1 ? 1 : p->tc_nder;
   dim3 grid(tc_ring_blocks(p, spin), p->mmax + 1);
@@ -1361,14 +1366,25 @@ cudaError_t launch_tcstart(const tl_plan *p, int which, int *bstart, float *stat
 #define CASE(n)                                                                                      \
   case n:                                                                                            \
     if (spin == 2)                                                                                   \
-      tcstart_kernel<n, true><<<grid, kComputeThreads, 0, s>>>(D, bstart, state, state_mid, ms);     \
+      tcstart_kernel<n, true><<<grid, kComputeThreads, 0, s>>>(D, bstart, state, state_mid, ms, tables);  \
     else                                                                                             \
-      tcstart_kernel<n, false><<<grid, kComputeThreads, 0, s>>>(D, bstart, state, state_mid, ms);    \
+      tcstart_kernel<n, false><<<grid, kComputeThreads, 0, s>>>(D, bstart, state, state_mid, ms, tables); \
     return cudaGetLastError();
     TL_TC_ORDERS(CASE)
 #undef CASE
   }
   return cudaErrorInvalidValue;
+}
+
+// Part tables that the kernels of a plan read beside the start table: none where a unit is one part, the
+// second half's where it is two, three where it is four. The potential alone runs in parts of its
+// own; in the persistent launch (tl_batch plans) it takes the plan's. At Nside 2048 / lmax 4096, order 4, a
+// table has 0.74 GB for T, 1.47 GB for Q/U and 0.34 GB for the potential; the time to fill them goes with the
+// part of the l range that they need.
+int tc_part_tables(const tl_plan *p, int which) {
+  const int mode = tc_mode(p->precision), nc = tc_cols(p->tc_nder);
+  const int own = tc_parts((which == 1 ? 1 : p->tc_nder) + 1, mode, nc), plan = tc_parts(p->tc_nder + 1, mode, nc);
+  return (p->tc_persistent && plan > own ? plan : own) - 1;
 }
 
 // Start-table bytes: the state of 128 rings (2 NJ + 1 words each) per unit.

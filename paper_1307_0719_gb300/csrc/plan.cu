@@ -287,7 +287,8 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
       float **sm = which == 0 ? &p->tc_sm0 : which == 1 ? &p->tc_smp : &p->tc_sm2;
       TRY_CUDA(dalloc((void **)bs, sizeof(int) * tc_start_units(p, which), B));
       TRY_CUDA(dalloc((void **)st, tc_start_state_bytes(p, which), B));
-      TRY_CUDA(dalloc((void **)sm, 3 * tc_start_state_bytes(p, which), B));
+      const int tables = tc_part_tables(p, which);
+      if (tables) TRY_CUDA(dalloc((void **)sm, tables * tc_start_state_bytes(p, which), B));
       TRY_CUDA(launch_tcstart(p, which, *bs, *st, *sm, 0));
     }
     TRY_CUDA(cudaDeviceSynchronize());
@@ -316,6 +317,11 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
 
 extern "C" tl_status tl_plan_create(int nside, int lmax, int order, int spins, int precision, int flags,
                                     tl_plan **out) {
+  return plan_create(nside, lmax, order, spins, precision, flags, 0, out);
+}
+
+tl_status tl::plan_create(int nside, int lmax, int order, int spins, int precision, int flags, int persistent,
+                          tl_plan **out) {
   if (!out) return TL_ERR_ARG;
   if (nside < 1 || nside > 8192 || (nside & (nside - 1)) != 0) return TL_ERR_ARG;
   if (lmax < 1 || lmax > 8 * nside) return TL_ERR_ARG;  // 8 nside: the paper's gradient band limit
@@ -343,6 +349,7 @@ extern "C" tl_status tl_plan_create(int nside, int lmax, int order, int spins, i
   }
   tl_plan *p = (tl_plan *)calloc(1, sizeof(tl_plan));
   if (!p) return TL_ERR_NOMEM;
+  p->tc_persistent = persistent;
   tl_status st = create_impl(nside, lmax, order, spins, precision, flags, p);
   if (st != TL_OK) {
     cudaDeviceSynchronize();
