@@ -298,9 +298,11 @@ tl_status tl_deflection_noalloc(int nside, int lmax, int precision, const double
  *   The persistent and graph modes need the lensing potential for every realisation
  *   (else TL_ERR_UNSUPPORTED); on non-tensor-core plans they run the loop.
  *   Arrays (host) of nreal device pointers, layouts as in tl_lens.
- *   tl_batch_autotune: times the persistent grid size and the ring-FFT batching
- *   on the given data (synchronises), keeps the fastest, and appends it to the file
- *   named by TAYLENS_TUNE_CACHE when set; tl_batch_create reads that file.
+ *   tl_batch_autotune: times what the batch leaves a choice of on the given data (synchronises), keeps
+ *   the fastest, and appends it to the file named by TAYLENS_TUNE_CACHE when set; tl_batch_create
+ *   reads that file. That is the persistent grid size where more than one block fits an SM (order 1),
+ *   and the batching of Bluestein's sub-transforms where rings take the general ring FFT
+ *   (Nside above 2048, or TAYLENS_RING_FFT=shared). The output maps may be written.
  */
 typedef struct tl_batch tl_batch;
 enum { TL_BATCH_LOOP = 0, TL_BATCH_PERSISTENT = 1, TL_BATCH_GRAPH = 2 };

@@ -9,8 +9,8 @@
 // from an atomic counter; ring FFTs and the gather then follow per realisation.
 // The whole sequence can be captured once in a CUDA graph and replayed. The
 // reference point is a plain per-realisation loop of tl_lens calls. An autotuner
-// times the persistent grid size and the ring-FFT batching on the caller's data
-// and keeps the choice (optionally in a cache file named by TAYLENS_TUNE_CACHE).
+// times the persistent grid size and the ring-FFT batching, where a batch has a choice of them, on the
+// caller's data and keeps the choice (optionally in a cache file named by TAYLENS_TUNE_CACHE).
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -382,7 +382,9 @@ extern "C" tl_status tl_batch_lens(tl_batch *b, int mode, const double *const *a
 }
 
 // Time candidate persistent grids and ring-FFT batching on the caller's data; keep
-// the fastest (and append it to TAYLENS_TUNE_CACHE when set). Synchronises.
+// the fastest (and append it to TAYLENS_TUNE_CACHE when set). Synchronises. Only what reaches a kernel is
+// timed: the batching where a plan has Bluestein rings on the general ring kernel (above Nside 2048, or with
+// TAYLENS_RING_FFT=shared), the grid where tensor memory leaves room for more than one CTA per SM.
 extern "C" tl_status tl_batch_autotune(tl_batch *b, const double *const *alm_T, const double *const *alm_E,
                                        const double *const *alm_B, const double *const *alm_phi,
                                        void *const *T_out, void *const *Q_out, void *const *U_out, void *stream) {
@@ -407,31 +409,37 @@ extern "C" tl_status tl_batch_autotune(tl_batch *b, const double *const *alm_T, 
     return TL_OK;
   };
   // 1. ring-FFT batching (one knob per group, all groups together)
-  float best = 1e30f;
-  int best_fb = 1;
-  for (int fb : {1, 4}) {
-    for (tl_plan *p : b->plans) p->fft_batch = fb;
-    float ms;
-    tl_status st = timeit(&ms);
-    if (st != TL_OK) return st;
-    if (ms < best) {
-      best = ms;
-      best_fb = fb;
+  bool batching = false;
+  for (const tl_plan *p : b->plans) batching = batching || ringfft_batch_choice(p);
+  if (batching) {
+    float best = 1e30f;
+    int best_fb = 1;
+    for (int fb : {1, 4}) {
+      for (tl_plan *p : b->plans) p->fft_batch = fb;
+      float ms;
+      tl_status st = timeit(&ms);
+      if (st != TL_OK) return st;
+      if (ms < best) {
+        best = ms;
+        best_fb = fb;
+      }
     }
+    for (tl_plan *p : b->plans) p->fft_batch = best_fb;
   }
-  for (tl_plan *p : b->plans) p->fft_batch = best_fb;
   // 2. persistent grid size (blocks per SM)
-  best = 1e30f;
-  int best_grid = b->grid;
   const int ctas = tc_persistent_ctas(b->plans[0]->tc_nder, b->precision);
-  for (int k : {ctas > 1 ? ctas / 2 : 1, ctas}) {
-    b->grid = nsm * k;
-    float ms;
-    tl_status st = timeit(&ms);
-    if (st != TL_OK) return st;
-    if (ms < best) {
-      best = ms;
-      best_grid = b->grid;
+  int best_grid = nsm * ctas;
+  if (ctas > 1) {
+    float best = 1e30f;
+    for (int k : {ctas / 2, ctas}) {
+      b->grid = nsm * k;
+      float ms;
+      tl_status st = timeit(&ms);
+      if (st != TL_OK) return st;
+      if (ms < best) {
+        best = ms;
+        best_grid = b->grid;
+      }
     }
   }
   b->grid = best_grid;

@@ -269,6 +269,7 @@ long long host_bluestein_layout(int nside, long long *off, int *ml, int *maxm);
 int host_twiddle_len(int nside, int maxm);
 void host_twiddles(int TW, double *tw);
 size_t ringfft_smem_bytes(const tl_plan *p);
+bool ringfft_batch_choice(const tl_plan *p);
 // ring-FFT launch groups (no allocation): fills groups[] and order[nrings]; returns
 // the number of groups, or -1 if there are more than TL_MAX_FFT_GROUPS
 // (of the rings with use[r] != 0 only, when use is given)

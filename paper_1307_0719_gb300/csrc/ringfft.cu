@@ -733,6 +733,15 @@ static int group_batch(const tl_plan *p, const FftGroup &g, bool reg) {
   if (p->fft_batch == 4) return s4 <= 227 * 1024 ? 4 : 1;
   return s4 <= 113 * 1024 ? 4 : 1;
 }
+// Whether a plan's ring FFTs depend on fft_batch (1 or 4)
+bool ringfft_batch_choice(const tl_plan *p) {
+  const bool sy = p->sy_ngroups > 0;
+  const FftGroup *groups = sy ? p->rest_groups : p->fft_groups;
+  for (int i = 0; i < (sy ? p->rest_ngroups : p->fft_ngroups); ++i)
+    if (groups[i].M > 0 && group_smem(p, groups[i], 4, false) <= 227 * 1024) return true;
+  return false;
+}
+
 // Upper bound over all rings (plan feasibility check): batch 1.
 size_t ringfft_smem_bytes(const tl_plan *p) {
   const size_t e2 = (p->precision == TL_FP64) ? 16 : 8;
