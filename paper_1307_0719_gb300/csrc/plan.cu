@@ -178,6 +178,11 @@ static tl_status create_impl(int nside, int lmax, int order, int spins, int prec
       p->rest_ngroups = host_fft_groups(nside, p->nrings, h.nphi.data(), ml.data(), p->rest_groups, order.data(),
                                         use.data());
       if (p->rest_ngroups < 0) return TL_ERR_UNSUPPORTED;
+      // The general kernel reads chirp spectra in bit-reversed order, which float plans keep for lengths other than
+      // 2^11 and 2^12 (blue_reg_lg below). No ring with such a length comes here: a ring that no grid fits is
+      // the belt (a power of two) or has more than 8190 pixels, so M >= 2^13.
+      for (int i = 0; i < p->rest_ngroups; ++i)
+        if (p->rest_groups[i].M >= 1 << 11 && p->rest_groups[i].M <= 1 << 12) return TL_ERR_UNSUPPORTED;
       TRY_CUDA(upload(&p->rest_rings, order, B));
     }
     const float *cw = host_synth_window(&p->sy_win);
