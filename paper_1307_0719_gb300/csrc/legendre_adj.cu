@@ -330,8 +330,8 @@ __global__ void __launch_bounds__(128) legendre_adj2_kernel(RingTable rt, const 
 // tests of the scale once every ring of the warp has reached 0, and the parity of l + m is that
 // of the position in the window (the spin-2 sums U1 and U2 change places once, at m = 1, instead of
 // being selected in every step). Every value is formed by the same operations in the same order.
-// Order 4, Nside 1024 / lmax 2048: spin 2 25.7 -> 16.6 ms, spin 0 with the potential 9.7 -> 7.8 ms (101 ->
-// about 62 instructions per ring and step at spin 2); at order 0, the whole analysis, 23.6 -> 14.2 ms.
+// Order 4, Nside 1024 / lmax 2048: spin 2 25.7 -> 16.6 ms, spin 0 with the potential 9.7 -> 7.8 ms (at
+// Nside 512 / lmax 1024 spin 2 issues 1.99 instead of 3.41 G warp instructions, 59 instead of 101 per ring, l and m); at order 0, the whole analysis, 23.6 -> 14.2 ms.
 
 template <int NDER, bool PHI>
 __global__ void __launch_bounds__(128) legendre_adj0_f32_kernel(RingTable rt, const double *__restrict__ lnorm0,

@@ -224,7 +224,7 @@ __device__ __forceinline__ void bf16_split2(float x0, float x1, uint32_t &hi, ui
 // Parts of the l range a unit is split into (sets of four compute warps on the same rings,
 // see run_blocks): 4 where a CTA fills the SM anyway and four sets of basis tiles fit the 512
 // columns, else 2 where two sets fit, else 1. (Two CTAs of two parts per SM for the potential: a
-// CTA of four parts has 544 threads of up to 120 registers, and only one fits.)
+// CTA of four parts has 608 threads, 96 registers each at order 4, and only one fits.)
 __host__ __device__ constexpr int tc_parts(int nj, int mode, int nc) {
   const int acc = nj * nc, aset = nj * (mode == kModeTf32x3 ? 16 : 8);
   return acc + 4 * aset <= 256 ? 2 : acc + 4 * aset <= 512 ? 4 : acc + 2 * aset <= 512 ? 2 : 1;
@@ -481,10 +481,11 @@ template <int NC, int NH> __host__ __device__ constexpr uint32_t xch_offset() {
 // accumulators unset).
 //
 // What bounds it: the tensor pipe takes one M = 128, K = 16 instruction per 46 cycles for any
-// N up to 64 (measured), ten per block at order 4, so a block cannot take less than 467 cycles;
+// N up to 64, ten per block at order 4, so a block cannot take less than 467 cycles;
 // at Nside 2048 / lmax 3000 it takes 820 in the loop (the issuing warp shares its scheduler with
-// compute warps that are 67% issue-active, and waits 240 cycles per two blocks) and 950 with the unit's
-// start, end and epilogue. Before (two parts, the tiles through the compute warps' registers, one
+// compute warps, and waits 240 cycles per two blocks) and 950 with the unit's
+// start, end and epilogue (isolated probes, and clock reads in a scratch copy of the kernel). Counters at Nside 512 /
+// lmax 1024: tensor pipe 31% active, SM 52% issue-active with 18.9 warps (two parts: 21%, 38% and 9.0). Before (two parts, the tiles through the compute warps' registers, one
 // lane per block): 1330. Spin 2 103.9 -> 73.0 ms, spin 0 with the potential 70.0 -> 51.5 ms (of which one
 // millisecond each from not storing the coefficients that every ring of a warp holds at zero).
 template <int NDER, int MODE, int NC, int NB, bool SPIN2, int NH>

@@ -564,7 +564,8 @@ static tl_status lens_fft(tl_plan *p, const void *const *planes, bool phi, cudaS
     jobs.resize(2);
     deflection_jobs(p, p->alpha, (char *)p->alpha + (size_t)p->elem * p->npix, il, jobs.data());
   }
-  // Jobs are packed two per transform in list order. Q and U of the same (j, k)
+  // The synthesis kernels take each map by itself (and sort them by plane); the general ring kernel packs
+  // jobs two per transform in list order. So Q and U of the same (j, k)
   // pair (similar magnitudes) and come first, an even count; then the T maps, which
   // pair within one coefficient plane j (the fold reads the row once for both),
   // left-overs across planes, the last one alone when their count is odd.

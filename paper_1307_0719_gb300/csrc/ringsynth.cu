@@ -30,7 +30,9 @@
 // ring's length the aliases are folded while staging (per map, since (m / L)^k is not a
 // function of m modulo the length).
 //
-// What bounds it: instruction issue. Sixteen T+Q/U realisations of order 4 take 118 ms at
+// What bounds it: instruction issue (Nside 2048 / lmax 3000: the belt 69% issue-active at 23 warps per SM, the caps
+// of H = 4096 67% and their two-grid form 78%, of H = 2048 60%, at 31 warps; DRAM below 45% of its copy
+// rate). Sixteen T+Q/U realisations of order 4 take 118 ms at
 // Nside 2048 / lmax 3000 and 10.4 ms at Nside 512 / lmax 1024, against 232 and 21.9 ms for packed
 // pairs of maps with Bluestein's convolution in the caps. One weight for a pixel and
 // its mirror image took 6 ms off at Nside 2048 (the cap kernels' instructions per map and pixel fell by
@@ -624,8 +626,9 @@ static cudaError_t synth_launch(const tl_plan *p, const SyGroup &g, const JobLis
 // serialization; the first waits for the stream as usual): otherwise every group ends in a partly empty
 // chip. What follows the last group is ordered after that group alone, in a captured graph above all,
 // so every block waits for the group before at its end: the groups then complete in order. The
-// blocks that wait have all been placed, and those they wait for have all started. Up to Nside 1024: sixteen skies at Nside 512 take
-// 10.0 instead of 10.6 ms, but at Nside 2048, where the ends weigh little, 109.7 instead of 107.6.
+// blocks that wait have all been placed, and those they wait for have all started. Up to Nside 1024: sixteen skies take 0.31 instead of
+// 0.40 ms at Nside 32, 0.91 for 1.12 at 128, 2.94 for 3.28 at 256, 10.4 for 11.0 at 512 and 37.9 for 39.1 at
+// 1024, but 120.2 for 117.8 at 2048, where the ends weigh little.
 cudaError_t launch_ring_synth(const tl_plan *p, JobList &jl, cudaStream_t s) {
   const double c = synth_power(p->lmax) / (double)(p->lmax + 1);
   for (int i = 0; i < jl.n; ++i) jl.job[i].scalef = (float)(jl.job[i].scale * pow(c, jl.job[i].k));
