@@ -156,7 +156,7 @@ template <int DIR> struct TwidTable {
   }
 };
 // or a table of six (q = 1, 2, 3, 4, 8, 12; DIR = +1), pass by pass, so that every other one is a single
-// product: a float transform's error falls by a seventh against four and products of up to three (1.40e-7 ->
+// product: a float transform's error is 9% below that of four and products of up to three (1.40e-7 ->
 // 1.28e-7 relative RMS on the belt rings at Nside 512 to 2048) at the same time. Three rows of L / 16 pairs, so that
 // a warp's loads are contiguous (the scattered entries of tw lie in up to 88 lines; all fifteen from a table
 // took 6% more of the whole synthesis at Nside 2048).
